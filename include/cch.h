@@ -33,7 +33,7 @@
  * stream).  Device buffers belong to the caller and must stay valid until
  * the stream reaches the call.  The library keeps one scratch workspace per
  * stream (device memory, grown on demand, reused by later calls on that
- * stream); cch_release_workspace() frees it.  Calls on one stream are
+ * stream; calls of small sets need none); cch_release_workspace() frees it.  Calls on one stream are
  * serialised by the stream; calls on different streams use different
  * workspaces and may overlap on the device.
  *
@@ -181,7 +181,8 @@ int cch_hull_stages(const void *points, int64_t n, int dtype, uint32_t opts,
  * number of stages (8).  cch_profile(0) stops recording.  cch_profile_stages(mask)
  * records only around the stages whose bit is set in mask (bit k: stage k;
  * the others read as 0), which keeps the events' own cost out of the rest
- * of the pipeline; mask 0 stops recording.
+ * of the pipeline; mask 0 stops recording.  Small sets are computed by one
+ * kernel each, outside these stages.
  */
 int cch_profile(int enable);
 int cch_profile_stages(uint32_t mask);
@@ -263,7 +264,7 @@ int cch_autotune_batched(const void *points, const int64_t *offsets, int32_t nse
                          int32_t *out_idx, int32_t *out_counts, void *stream, int32_t reps,
                          cch_tune_params *best);
 
-/* Bytes of device scratch one cch_hull call of this size uses. */
+/* Bytes of device scratch one cch_hull call of this size uses at most. */
 size_t cch_workspace_bytes(int64_t n, int dtype);
 
 /* Free every cached workspace and the servers' pooled pinned host buffers

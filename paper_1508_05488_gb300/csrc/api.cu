@@ -44,7 +44,6 @@ struct Layout {
   size_t total = 0;
   size_t ctl_bytes = 0;                  // ctl + ctr (cleared each call)
   size_t status_off = 0, status_bytes = 0;   // look-back words (cleared on epoch wrap)
-  size_t sets_off = 0;
   Ws w{};
 };
 
@@ -84,8 +83,6 @@ Layout layout(const Dims& d, char* base) {
   L.w.blk_tail = (int32_t*)take(4 * (size_t)d.max_chain_blks);
   L.w.out_start = (uint32_t*)take(4 * (4 * (size_t)d.nsets + 1));
   L.w.stairs = (uint32_t*)take(4 * 4 * (size_t)kStairB * d.nsets);
-  L.sets_off = o;
-  take(sizeof(SetDesc) * (size_t)d.nsets);
   L.total = o;
   return L;
 }
@@ -95,9 +92,10 @@ struct Workspace {
   size_t bytes = 0;
   Dims cap{};
   uint32_t epoch = 0;
-  SetDesc* host_sets = nullptr;      // pinned staging of the set table
-  size_t host_sets_cap = 0;
-  cudaEvent_t sets_done = nullptr;   // staging buffer free again
+  char* host_tab = nullptr;          // pinned staging of a batch's tables
+  char* dev_tab = nullptr;           // their device copy
+  size_t tab_bytes = 0;              // size of both
+  cudaEvent_t tab_done = nullptr;    // staging buffer free again
   void* h2d = nullptr;               // device copy of host points (cch_hull_host)
   size_t h2d_bytes = 0;
   int32_t* dcount = nullptr;         // device counts (cch_hull_host)
@@ -140,10 +138,8 @@ bool fits(const Dims& c, const Dims& d) {
   return d.N <= c.N && d.nsets <= c.nsets && d.nchunk1 <= c.nchunk1 && d.ntile2 <= c.ntile2;
 }
 
-// Get (or grow) the workspace of `stream` for dims `d`.  Called with g_mu held.
-int acquire(cudaStream_t stream, const Dims& d, Workspace** out) {
-  Workspace*& ws = g_ws[stream];
-  if (!ws) ws = new Workspace();
+// Grow the workspace `ws` of `stream` to dims `d`.  Called with g_mu held.
+int acquire(cudaStream_t stream, const Dims& d, Workspace* ws) {
   if (!ws->dev || !fits(ws->cap, d)) {
     Dims c = d;
     if (ws->dev) {   // grow by at least 1.5x to amortise
@@ -167,7 +163,6 @@ int acquire(cudaStream_t stream, const Dims& d, Workspace** out) {
     ws->cap = c;
     ws->epoch = 0;
   }
-  *out = ws;
   return CCH_OK;
 }
 
@@ -178,20 +173,81 @@ int a1_target(int dtype) {
 
 int grid_cap() { return sm_count() * 4; }
 
-// Launch the whole pipeline for the job; `sets_host` is the set table for a
-// batch (nullptr for a single set).  `stages` hooks the stage extraction.
 struct StageOut {
   int32_t* r1_idx;
   int32_t* r1_region;
   int32_t* spa_idx;
 };
 
-int run(Job& j, const std::vector<SetDesc>* sets_host, cudaStream_t stream, StageOut* stages,
-        Workspace** ws_out) {
+// The sets of a batch: the pipeline's, and the small ones of k_set by class.
+struct Batch {
+  std::vector<SetDesc> sets;
+  std::vector<SetItem> items[kSetClasses];
+};
+
+// Copy a batch's tables (small sets by class, then the pipeline's sets) to the
+// device, and launch k_set on the small ones.  Called with g_mu held; returns
+// a status, the kernels launched are added to *nk.
+int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int* nk) {
+  size_t ibytes = 0;
+  for (const auto& v : b.items) ibytes += sizeof(SetItem) * v.size();
+  const size_t sets_off = (ibytes + 63) / 64 * 64;
+  const size_t bytes = sets_off + sizeof(SetDesc) * b.sets.size();
+  if (!ws->tab_done && cudaEventCreateWithFlags(&ws->tab_done, cudaEventDisableTiming) != cudaSuccess) return CCH_ERR_CUDA;
+  if (cudaEventSynchronize(ws->tab_done) != cudaSuccess) return CCH_ERR_CUDA;
+  if (ws->tab_bytes < bytes) {
+    if (cudaStreamSynchronize(stream) != cudaSuccess) return CCH_ERR_CUDA;   // earlier calls read the old copy
+    if (ws->host_tab) cudaFreeHost(ws->host_tab);
+    if (ws->dev_tab) cudaFree(ws->dev_tab);
+    ws->host_tab = ws->dev_tab = nullptr;
+    ws->tab_bytes = 0;
+    const size_t cap = bytes + bytes / 2;
+    if (cudaMallocHost(&ws->host_tab, cap) != cudaSuccess || cudaMalloc(&ws->dev_tab, cap) != cudaSuccess) {
+      cudaGetLastError();
+      if (ws->host_tab) cudaFreeHost(ws->host_tab);
+      ws->host_tab = ws->dev_tab = nullptr;
+      return CCH_ERR_NOMEM;
+    }
+    ws->tab_bytes = cap;
+  }
+  size_t o = 0;
+  for (const auto& v : b.items) {
+    if (!v.empty()) memcpy(ws->host_tab + o, v.data(), sizeof(SetItem) * v.size());
+    o += sizeof(SetItem) * v.size();
+  }
+  if (!b.sets.empty()) memcpy(ws->host_tab + sets_off, b.sets.data(), sizeof(SetDesc) * b.sets.size());
+  if (cudaMemcpyAsync(ws->dev_tab, ws->host_tab, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
+  if (cudaEventRecord(ws->tab_done, stream) != cudaSuccess) return CCH_ERR_CUDA;
+  const SetItem* items = reinterpret_cast<const SetItem*>(ws->dev_tab);
+  o = 0;
+  for (int c = 0; c < kSetClasses; c++) o += b.items[c].size();
+  for (int c = kSetClasses - 1; c >= 0; c--) {     // the largest sets first
+    o -= b.items[c].size();
+    *nk += launch_set(j, c, items + o, (int)b.items[c].size(), stream);
+  }
+  j.sets = reinterpret_cast<const SetDesc*>(ws->dev_tab + sets_off);
+  return CCH_OK;
+}
+
+// Launch the whole call: k_set on a batch's small sets, the pipeline on the
+// others (`batch` nullptr: the single set of j.one).  `stages` hooks the
+// stage extraction.
+int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Workspace** ws_out) {
   Dims d = make_dims(j.N, j.nsets, j.nchunk1, j.ntile2);
   std::lock_guard<std::mutex> lk(g_mu);
-  Workspace* ws = nullptr;
-  int st = acquire(stream, d, &ws);
+  Workspace*& slot = g_ws[stream];
+  if (!slot) slot = new Workspace();
+  Workspace* ws = slot;
+  int nk = 0;
+  if (batch) {
+    const int st = start_batch(j, *batch, ws, stream, &nk);
+    if (st != CCH_OK) return st;
+    if (batch->sets.empty()) {
+      g_launches += (uint64_t)nk;
+      return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
+    }
+  }
+  int st = acquire(stream, d, ws);
   if (st != CCH_OK) return st;
   Layout L = layout(ws->cap, ws->dev);
   if (++ws->epoch > 0xFFFu) {
@@ -200,27 +256,10 @@ int run(Job& j, const std::vector<SetDesc>* sets_host, cudaStream_t stream, Stag
   }
   j.epoch = ws->epoch;
   if (cudaMemsetAsync(ws->dev, 0, L.ctl_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
-  if (sets_host) {
-    size_t bytes = sizeof(SetDesc) * sets_host->size();
-    if (ws->host_sets_cap < sets_host->size()) {
-      if (ws->host_sets) { cudaEventSynchronize(ws->sets_done); cudaFreeHost(ws->host_sets); }
-      if (cudaMallocHost(&ws->host_sets, bytes) != cudaSuccess) { ws->host_sets = nullptr; ws->host_sets_cap = 0; return CCH_ERR_NOMEM; }
-      ws->host_sets_cap = sets_host->size();
-      if (!ws->sets_done) cudaEventCreateWithFlags(&ws->sets_done, cudaEventDisableTiming);
-    } else if (ws->sets_done) {
-      cudaEventSynchronize(ws->sets_done);
-    }
-    memcpy(ws->host_sets, sets_host->data(), bytes);
-    SetDesc* dsets = reinterpret_cast<SetDesc*>(ws->dev + L.sets_off);
-    if (cudaMemcpyAsync(dsets, ws->host_sets, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
-    cudaEventRecord(ws->sets_done, stream);
-    j.sets = dsets;
-  }
   if (stages) { j.r1_idx = stages->r1_idx; j.r1_region = stages->r1_region; }
   Launch La{stream, grid_cap(), j.tune.cls_per_sm * sm_count()};
   ProfRec rec{};
   cudaEvent_t* ev = prof_begin(rec);
-  int nk = 0;
   // event k marks the start of stage k (and the end of stage k - 1)
   auto mark = [&](int k) {
     if (ev && ((rec.mask >> k) & 1u || (k > 0 && (rec.mask >> (k - 1)) & 1u))) cudaEventRecord(ev[k], stream);
@@ -283,13 +322,29 @@ Job single_job(const void* points, int64_t n, int dtype, int32_t* out_idx, int32
   j.nchunk3 = n > 0 ? (int32_t)((stairs_sample(n, j.tune) + kStairChunk - 1) / kStairChunk) : 0;
   j.nchunkP = (j.ntile2 + kPlanTiles - 1) / kPlanTiles;
   j.sets = nullptr;
-  j.one = SetDesc{0, n, 0, nch, 0, j.ntile2, 0, j.nchunk3, 0, j.nchunkP};
+  j.one = SetDesc{0, n, 0, nch, 0, j.ntile2, 0, j.nchunk3, 0, j.nchunkP, 0};
   j.out_idx = out_idx;
   j.out_counts = out_count;
   return j;
 }
 
-// ------------------------------------------------ float32 SoA input
+// A single set small enough for k_set: one launch, no workspace.
+Job set_job(const void* points, const float* ys, int64_t n, int dtype, int32_t* out_idx, int32_t* out_count) {
+  Job j{};
+  j.pts = points;
+  j.ys = ys;
+  j.N = n;
+  j.nsets = 1;
+  j.dtype = dtype;
+  j.out_idx = out_idx;
+  j.out_counts = out_count;
+  return j;
+}
+
+int run_set(const Job& j, cudaStream_t stream) {
+  g_launches += (uint64_t)launch_set(j, set_class(j.N), nullptr, 1, stream);
+  return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
+}
 
 }  // namespace
 
@@ -321,6 +376,7 @@ int cch_hull(const void* points, int64_t n, int dtype, int32_t* out_idx, int32_t
              void* stream) {
   int st = check_common(points, n, dtype, out_idx, out_count);
   if (st != CCH_OK) return st;
+  if (n <= kSetOne) return run_set(set_job(points, nullptr, n, dtype, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(points, n, dtype, out_idx, out_count, 0);
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
@@ -335,7 +391,7 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
   if (N > 0x7FFFFFFFll) return CCH_ERR_RANGE;
   if (N > 0 && !points) return CCH_ERR_INVALID;
   if ((uintptr_t)points % (dtype == CCH_F64 ? 16 : 8)) return CCH_ERR_INVALID;
-  std::vector<SetDesc> sets(nsets);
+  Batch batch;
   const Tune tune = tune_for(dtype, N, nsets);
   int target = a1_target(dtype);
   int64_t len = std::max<int64_t>(tune.a1_len_min, ((N + target - 1) / std::max(target, 1) + 1023) / 1024 * 1024);
@@ -345,11 +401,17 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
     int64_t n = offsets[s + 1] - offsets[s];
     if (n < 0) return CCH_ERR_INVALID;
     if (n > kMaxSetPoints) return CCH_ERR_RANGE;
+    const int cls = set_class(n);
+    if (cls >= 0) {
+      batch.items[cls].push_back(SetItem{offsets[s], (int32_t)n, s});
+      continue;
+    }
     int32_t c = (int32_t)((n + len - 1) / len);
     int32_t t = (int32_t)((n + ct - 1) / ct);
-    int32_t c3 = n > 0 ? (int32_t)((stairs_sample(n, tune) + kStairChunk - 1) / kStairChunk) : 0;
+    int32_t c3 = (int32_t)((stairs_sample(n, tune) + kStairChunk - 1) / kStairChunk);
     int32_t cp = (t + kPlanTiles - 1) / kPlanTiles;
-    sets[s] = SetDesc{offsets[s], n, (int32_t)nch, c, (int32_t)nt, t, (int32_t)n3, c3, (int32_t)np_, cp};
+    batch.sets.push_back(
+        SetDesc{offsets[s], n, (int32_t)nch, c, (int32_t)nt, t, (int32_t)n3, c3, (int32_t)np_, cp, s});
     nch += c;
     nt += t;
     n3 += c3;
@@ -358,7 +420,7 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
   Job j{};
   j.pts = points;
   j.N = N;
-  j.nsets = nsets;
+  j.nsets = (int32_t)batch.sets.size();
   j.dtype = dtype;
   j.tune = tune;
   j.nchunk1 = (int32_t)nch;
@@ -368,7 +430,7 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
   j.chunk1_len = len;
   j.out_idx = out_idx;
   j.out_counts = out_counts;
-  return run(j, &sets, (cudaStream_t)stream, nullptr, nullptr);
+  return run(j, &batch, (cudaStream_t)stream, nullptr, nullptr);
 }
 
 int cch_hull_host(const void* points_host, int64_t n, int dtype, int32_t* out_idx_host,
@@ -424,6 +486,7 @@ int cch_hull_f32soa(const float* x, const float* y, int64_t n, int32_t* out_idx,
   if (n < 0 || !out_idx || !out_count || (n > 0 && (!x || !y))) return CCH_ERR_INVALID;
   if ((((uintptr_t)x | (uintptr_t)y) & 3u) != 0) return CCH_ERR_INVALID;
   if (n > kMaxSetPoints) return CCH_ERR_RANGE;
+  if (n <= kSetOne) return run_set(set_job(x, y, n, DT_F32, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(x, n, DT_F32, out_idx, out_count, 0);
   j.ys = y;
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
@@ -544,8 +607,9 @@ void cch_release_workspace(void) {
   for (auto& kv : g_ws) {
     Workspace* ws = kv.second;
     if (ws->dev) cudaFree(ws->dev);
-    if (ws->host_sets) cudaFreeHost(ws->host_sets);
-    if (ws->sets_done) cudaEventDestroy(ws->sets_done);
+    if (ws->host_tab) cudaFreeHost(ws->host_tab);
+    if (ws->dev_tab) cudaFree(ws->dev_tab);
+    if (ws->tab_done) cudaEventDestroy(ws->tab_done);
     if (ws->h2d) cudaFree(ws->h2d);
     if (ws->dcount) cudaFree(ws->dcount);
     if (ws->didx) cudaFree(ws->didx);

@@ -2,7 +2,8 @@
 // pipeline (sm_103a).  Nothing here is visible through the C ABI.
 //
 // Pipeline (Sec. 2.1, steps 1-7), every stage a kernel, every set of points a
-// "set" (a single hull is a batch of one):
+// "set" (a single hull is a batch of one).  Small sets are computed whole by
+// one CTA each (k_set.cu, hull_block.cuh); the others take the pipeline:
 //   a1  k_extremes      four lexicographic extremes + edge set-up (step 1)
 //       k_stairs        dominance tables and box from a sample of each set;
 //                       its sample pass runs during a1's tail
@@ -148,6 +149,23 @@ struct SetDesc {
   int32_t nchunk3;      // stairs chunks of this set
   int32_t chunkP;       // first survivor-count chunk (kPlanTiles a2 tiles each)
   int32_t nchunkP;      // survivor-count chunks of this set
+  int32_t id;           // index of the set in the caller's batch (its output count)
+};
+
+// Sets of a batch of at most kSetMax points are computed whole by one CTA
+// each (k_set) and take no part in the pipeline below; a call of one set goes
+// there up to kSetOne points.  One CTA per set fills the chip when there are
+// many (600 sets of 16000 points: 0.20 / 0.21 / 0.81 ms on squares, disks and
+// circles, 0.57 / 0.73 / 1.76 in the pipeline); alone it is one SM against all
+// of them: 8000 points take 40 / 50 / 120 us there and 61 / 84 / 216 in the
+// pipeline, 16000 points 63 / 65 / 242 against 63 / 103 / 155.
+constexpr int kSetMax = 16383;
+constexpr int kSetOne = 12287;
+constexpr int kSetClasses = 4;
+struct SetItem {
+  int64_t off;          // first point, and first output slot
+  int32_t n;
+  int32_t id;           // index of the set in the caller's batch
 };
 
 // Per-call launch description.  A single hull carries its descriptor inline;
@@ -949,6 +967,8 @@ struct Launch {
 };
 
 // Each returns the number of kernels it launched.
+int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
+int launch_set(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st);   // items null: the one set
 int launch_extremes(const Job& j, const Ws& w, const Launch& L);
 int launch_stairs(const Job& j, const Ws& w, const Launch& L);
 int launch_classify(const Job& j, const Ws& w, const Launch& L);

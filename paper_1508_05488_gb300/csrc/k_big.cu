@@ -125,12 +125,12 @@ __device__ void plan_chain(const Job& j, const Ws& w) {
       const SetCtl& c = w.ctl[s];
       const uint32_t degen_all = (SF_DEGEN0 * 15u);
       if (c.status != 0) {
-        if (r == 0) j.out_counts[s] = c.status;
+        if (r == 0) j.out_counts[sd.id] = c.status;
       } else if (sd.n == 0) {
-        if (r == 0) j.out_counts[s] = 0;
+        if (r == 0) j.out_counts[sd.id] = 0;
       } else if ((c.flags & degen_all) == degen_all) {
         // every point identical: the hull is the single point E1
-        if (r == 0) { j.out_idx[sd.off] = (int32_t)c.eidx[0]; j.out_counts[s] = 1; }
+        if (r == 0) { j.out_idx[sd.off] = (int32_t)c.eidx[0]; j.out_counts[sd.id] = 1; }
       } else if (!(c.flags & (SF_DEGEN0 << r))) {
         uint32_t L = c.s2[r] + 2;
         tb = (L + kChainBlk - 1) / kChainBlk;

@@ -19,57 +19,9 @@
 //  k_output       stable compaction of the surviving positions of the four
 //                 chains of a set (each without its last point) into out_idx.
 #include "cch_internal.cuh"
+#include "chain.cuh"
 
 namespace cch {
-
-template <int DT>
-struct PT;
-template <>
-struct PT<DT_F64> { using T = double2; };
-template <>
-struct PT<DT_I32> { using T = int2; };
-
-template <int DT>
-__device__ __forceinline__ bool same_pt(const typename PT<DT>::T& a, const typename PT<DT>::T& b) {
-  return a.x == b.x && a.y == b.y;   // value equality: -0.0 == +0.0
-}
-
-// Merge two adjacent convex chains given by (head, tail) into the left one.
-// Links, flags, points and orientation go through the accessor (shared or
-// global memory).
-template <class A>
-__device__ void merge_chains(A& acc, int& hl, int& tl, int hr, int tr) {
-  if (hr < 0) return;
-  if (hl < 0) { hl = hr; tl = tr; return; }
-  int a = tl, b = hr;
-  for (;;) {
-    bool moved = false;
-    while (a != hl && acc.orient(acc.prv(a), a, b) <= 0) {
-      acc.kill(a);
-      a = acc.prv(a);
-      moved = true;
-    }
-    while (b != tr && acc.orient(a, b, acc.nxt(b)) <= 0) {
-      acc.kill(b);
-      b = acc.nxt(b);
-      moved = true;
-    }
-    if (!moved) break;
-  }
-  acc.link(a, b);
-  tl = tr;
-}
-
-// Orientation of three chain points: float64 through the FP32 filter on
-// their views (when the set's coordinates allow), then exactly; int32
-// exactly in 64/128-bit integers.
-template <int DT>
-__device__ __forceinline__ int orient_chain(const typename PT<DT>::T& a, const typename PT<DT>::T& b,
-                                            const typename PT<DT>::T& c, float4 A, float4 B, float4 C,
-                                            bool flag) {
-  if constexpr (DT == DT_F64) return orient_f64_split(a, b, c, A, B, C, flag);
-  else return orient_i32(a.x, a.y, b.x, b.y, c.x, c.y, flag);
-}
 
 template <int DT>
 struct SmemAcc {
@@ -116,7 +68,6 @@ __device__ __forceinline__ void cp_async_copy(void* dst, const void* src) {
   else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(d), "l"(src) : "memory");
 }
 
-constexpr int kPeelRounds = 48;   // peeling rounds before the stack-and-merge fallback
 
 // Exclusive prefix sum of one value per thread over the CTA; sh[kWarps]
 // receives the total.  Ends with the CTA synchronised.
@@ -171,7 +122,7 @@ __device__ void chain_set_output(const Job& j, const Ws& w, const SetDesc& sd, i
     for (uint32_t k = threadIdx.x; k < nr; k += kThreads) j.out_idx[sd.off + off + k] = (int32_t)__ldcg(src + k);
     off += nr;
   }
-  if (threadIdx.x == 0) j.out_counts[s] = (int32_t)off;
+  if (threadIdx.x == 0) j.out_counts[sd.id] = (int32_t)off;
 }
 
 template <int DT>
@@ -409,7 +360,7 @@ __global__ void __launch_bounds__(kThreads) k_output(Job j, Ws w) {
     if (blockIdx.x == 0) {
       const int err = (int)ld_acq_u32(w.ctr + CT_ERR);
       if (err != 0)
-        for (int s = threadIdx.x; s < j.nsets; s += kThreads) j.out_counts[s] = err;
+        for (int s = threadIdx.x; s < j.nsets; s += kThreads) j.out_counts[get_set(j, s).id] = err;
     }
     return;
   }
@@ -471,7 +422,7 @@ __global__ void __launch_bounds__(kThreads) k_output(Job j, Ws w) {
       }
       if (lane == 0) {
         sh_excl = excl;
-        if (tile == last) j.out_counts[s] = (int32_t)(excl + agg);
+        if (tile == last) j.out_counts[sd.id] = (int32_t)(excl + agg);
       }
     }
     __syncthreads();
@@ -498,7 +449,7 @@ __global__ void __launch_bounds__(kThreads) k_output(Job j, Ws w) {
     __threadfence();
     const int err = (int)ld_acq_u32(w.ctr + CT_ERR);
     if (err != 0)
-      for (int s = threadIdx.x; s < j.nsets; s += kThreads) j.out_counts[s] = err;
+      for (int s = threadIdx.x; s < j.nsets; s += kThreads) j.out_counts[get_set(j, s).id] = err;
   }
 }
 

@@ -148,7 +148,7 @@ extern "C" int cch_hull_noalloc(const void* points, int64_t n, int dtype, int32_
   j.nchunk3 = n > 0 ? (int32_t)((stairs_sample(n, j.tune) + kStairChunk - 1) / kStairChunk) : 0;
   j.nchunkP = (j.ntile2 + kPlanTiles - 1) / kPlanTiles;
   j.sets = nullptr;
-  j.one = SetDesc{0, n, 0, j.nchunk1, 0, j.ntile2, 0, j.nchunk3, 0, j.nchunkP};
+  j.one = SetDesc{0, n, 0, j.nchunk1, 0, j.ntile2, 0, j.nchunk3, 0, j.nchunkP, 0};
 
   // set-up, once per device with that device current: the array's address
   if (!g_na_ptr[dev]) {
