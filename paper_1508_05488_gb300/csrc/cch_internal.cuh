@@ -67,7 +67,11 @@ constexpr int kStairChunk = 2048;      // sample points per k_stairs CTA (eight 
 constexpr int kStairLB = 512;          // buckets per region of a k_stairs CTA's own table
 constexpr int64_t kStairMin = 8192;    // smallest sample of a set
 constexpr int kPlanTiles = 64;         // a2 tiles per survivor-count chunk
-constexpr int kGatherSplit = 8;        // gather CTAs per chunk (all of them move a dense chunk)
+// Gather CTAs per chunk (all of them move a dense chunk): a warp moves its
+// sub-slots one after the other, so few chunks are split finely (circle of 2M
+// points, 16 chunks: 72 us at 8); a batch, with a chunk per small set at least,
+// takes 8.
+constexpr int kGatherSplit = 8, kGatherSplitMax = 64;
 constexpr int kGatherDense = 8192;     // survivors from which a chunk counts as dense
 // a1 reads the last kL2KeepBytes of every set without the evict-first hint,
 // so that they are still in L2 when k_stairs samples them (its sample is the

@@ -1417,12 +1417,14 @@ __global__ void __launch_bounds__(kClsBlock, 2) k_classify(Job j, Ws w) {
 __global__ void __launch_bounds__(kThreads) k_gather(Job j, Ws w) {
   griddep_enter();
   constexpr int kChunkSub = kPlanTiles * kClsConsumers;     // sub-slots of a chunk
-  constexpr int kPartSub = kChunkSub / kGatherSplit;         // sub-slots of a part of a dense chunk
+  static_assert(kChunkSub / kGatherSplitMax % kWarps == 0, "whole sub-slots per warp");
+  const int split = (int)gridDim.x / max(j.nchunkP, 1);
+  const int part_sub = kChunkSub / split;                    // sub-slots of a part of a dense chunk
   __shared__ uint32_t sh_tot[4], sh_cpre[4], sh_ct;
   __shared__ uint32_t wtot[kWarps][4], wpre[kWarps][4];
   __shared__ int sh_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int chunk = blockIdx.x / kGatherSplit, part = blockIdx.x % kGatherSplit;
+  const int chunk = blockIdx.x / split, part = blockIdx.x % split;
   int s = 0;
   if (j.sets) {
     int lo = 0, hi = j.nsets - 1;
@@ -1467,14 +1469,14 @@ __global__ void __launch_bounds__(kThreads) k_gather(Job j, Ws w) {
     }
     __syncthreads();
     // A chunk with few survivors is moved by its first CTA alone; a dense
-    // one by all kGatherSplit CTAs of the chunk, each a part of its
+    // one by all `split` CTAs of the chunk, each a part of its
     // sub-slots (the survivors of the earlier parts are counted first).
     const bool dense = sh_ct >= (uint32_t)kGatherDense;
     if (dense || part == 0) {                          // uniform across the CTA
       const int64_t nsub = (int64_t)sd.ntile2 * kClsConsumers;
       const int64_t cs0 = (int64_t)lc * kChunkSub;
-      const int64_t a = dense ? cs0 + (int64_t)part * kPartSub : cs0;
-      const int per_warp = (dense ? kPartSub : kChunkSub) / kWarps;
+      const int64_t a = dense ? cs0 + (int64_t)part * part_sub : cs0;
+      const int per_warp = (dense ? part_sub : kChunkSub) / kWarps;
       const int64_t g0 = a + warp * per_warp;
       const int64_t g1 = min(g0 + per_warp, nsub);
       const uint64_t* tc = w.tcnt + (size_t)sd.tile2 * kClsConsumers;
@@ -1611,7 +1613,10 @@ int launch_stairs(const Job& j, const Ws& w, const Launch& L) {
 }
 
 int launch_gather(const Job& j, const Ws& w, const Launch& L) {
-  launch_pdl(k_gather, (j.nchunkP < 1 ? 1 : j.nchunkP) * kGatherSplit, kThreads, 0, L.stream, j, w);
+  const int chunks = j.nchunkP < 1 ? 1 : j.nchunkP;
+  int split = kGatherSplit;
+  while (split < kGatherSplitMax && chunks * split <= 1024) split *= 2;
+  launch_pdl(k_gather, chunks * split, kThreads, 0, L.stream, j, w);
   return 1;
 }
 
