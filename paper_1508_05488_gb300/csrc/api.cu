@@ -83,6 +83,9 @@ Layout layout(const Dims& d, char* base) {
   L.w.blk_tail = (int32_t*)take(4 * (size_t)d.max_chain_blks);
   L.w.out_start = (uint32_t*)take(4 * (4 * (size_t)d.nsets + 1));
   L.w.stairs = (uint32_t*)take(4 * 4 * (size_t)kStairB * d.nsets);
+  L.w.sv_hdr = (SieveHdr*)take(sizeof(SieveHdr));
+  L.w.sv_tab = (float4*)take(sieve_table_bytes());
+  L.w.sv_cnt = (uint32_t*)take(4 * (size_t)kSvMaxUnits);
   L.total = o;
   return L;
 }
@@ -264,6 +267,7 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   auto mark = [&](int k) {
     if (ev && ((rec.mask >> k) & 1u || (k > 0 && (rec.mask >> (k - 1)) & 1u))) cudaEventRecord(ev[k], stream);
   };
+  if (j.sieve.nunit) nk += launch_sieve(j, L.w, stream);
   mark(0);
   nk += launch_extremes(j, L.w, La);
   mark(1);
@@ -378,6 +382,7 @@ int cch_hull(const void* points, int64_t n, int dtype, int32_t* out_idx, int32_t
   if (st != CCH_OK) return st;
   if (n <= kSetOne) return run_set(set_job(points, nullptr, n, dtype, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(points, n, dtype, out_idx, out_count, 0);
+  j.sieve = sieve_set(0, n, dtype, sm_count());
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
 
@@ -489,6 +494,7 @@ int cch_hull_f32soa(const float* x, const float* y, int64_t n, int32_t* out_idx,
   if (n <= kSetOne) return run_set(set_job(x, y, n, DT_F32, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(x, n, DT_F32, out_idx, out_count, 0);
   j.ys = y;
+  j.sieve = sieve_set(0, n, DT_F32, sm_count());
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
 

@@ -136,6 +136,7 @@ enum : int {
   CT_SPA_TOTAL,
   CT_CHAIN_TOTAL,
   CT_OUT_TOTAL,
+  CT_SIEVED,                           // the set was finished by the sieve path: the pipeline's kernels leave
   CT_ERR,                              // first device error (negative status)
   CT_COUNT
 };
@@ -172,6 +173,22 @@ struct SetItem {
   int32_t id;           // index of the set in the caller's batch
 };
 
+// A set of the sieve (k_sieve.cu): nunit units of len consecutive points.
+struct SieveSet {
+  int64_t off, n;
+  int64_t cap;          // most points a sieved set may keep (by the sample's estimate)
+  int64_t len;          // points per unit
+  int32_t nunit;
+  int32_t pre;          // points at the head of every unit that are prefetched
+};
+constexpr int kSvMaxUnits = 5120;
+// Device side of it: the maps of the bands (of Y: s[0] Y + o[0], of X: s[1] X +
+// o[1]), whether the sieve runs (mode) and the number of listed points.
+struct alignas(16) SieveHdr {
+  float s[2], o[2];
+  uint32_t mode, n;
+};
+
 // Per-call launch description.  A single hull carries its descriptor inline;
 // a batch points at a device array.
 struct Job {
@@ -190,6 +207,7 @@ struct Job {
   Tune tune;            // run-time choices (the same results with any valid choice)
   const SetDesc* sets;  // device array, or nullptr -> use `one`
   SetDesc one;
+  SieveSet sieve;       // nunit 0: the call does not sieve
   int32_t* out_idx;     // device
   int32_t* out_counts;  // device, [nsets]
   int32_t* r1_idx;      // stage hook (set 0, or nullptr): round-1 survivors, region-major
@@ -279,6 +297,9 @@ struct Ws {
   uint32_t* out_start;       // [4 nsets + 1] first output tile of (set, region)
   uint64_t* st_out;          // [max_out_tiles]
   uint32_t* stairs;          // [nsets][4][kStairB] bucket minima, then prefix minima
+  SieveHdr* sv_hdr;          // the sieve's header, band table and listed points per unit
+  float4* sv_tab;
+  uint32_t* sv_cnt;
 };
 
 // Chain slots of (set s, region r) when the region's records start at `rbase`
@@ -946,20 +967,45 @@ __device__ __forceinline__ void griddep_enter() { asm volatile("griddepcontrol.w
 // so k_stairs completes after a1 and a2's wait covers both.
 __device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Whether the sieve takes the set (k_sieve.cu).  The flag is written by
+// k_refine, which k_set waits for before it releases the pipeline.
+__device__ __forceinline__ bool sieved(const Ws& w) { return *(volatile const uint32_t*)(w.ctr + CT_SIEVED) != 0; }
+// The same at the start of a kernel of the pipeline, before its griddep_enter:
+// each starts when every CTA of the kernel before it has left or released it,
+// so the flag is there.  Where it is set the kernel has nothing to do: it lets
+// its successor start at once, and one CTA waits, so that the kernel still
+// completes after the one before it.  These nine launches run beside k_set and
+// add 5 us to a call where each waiting for the last one's end added 14.
+__device__ __forceinline__ bool sieved_leave(const Ws& w) {
+  if (!sieved(w)) return false;
+  griddep_release();
+  if (blockIdx.x == 0) griddep_enter();
+  return true;
+}
+
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args... args) {
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem,
+                                      cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              Args... args) {
+  return launch_pdl_cluster(kernel, grid, block, 1, smem, st, args...);
 }
 
 // ------------------------------------------------------------ launchers
@@ -973,6 +1019,10 @@ struct Launch {
 // Each returns the number of kernels it launched.
 int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
 int launch_set(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st);   // items null: the one set
+int launch_set_list(const Job& j, const Ws& w, cudaStream_t st);   // the sieve's listed points
+SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);
+size_t sieve_table_bytes();
+int launch_sieve(const Job& j, const Ws& w, cudaStream_t st);
 int launch_extremes(const Job& j, const Ws& w, const Launch& L);
 int launch_stairs(const Job& j, const Ws& w, const Launch& L);
 int launch_classify(const Job& j, const Ws& w, const Launch& L);

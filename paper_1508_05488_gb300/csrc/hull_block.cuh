@@ -56,6 +56,8 @@ struct BlkSmem {
   uint32_t w32[2][T / 32];
   uint32_t n[4];             // list lengths
   unsigned long long s2;     // SPA survivors per region, 16 bits each
+  uint32_t hn, hb;           // the hull's vertices and the list that holds them (0: a, 1: b)
+  uint32_t close;            // candidate number of the point that closes the polygon
 };
 
 // Sort key and SPA value of a point of region r (0..3), Table 1 / Fig. 2.
@@ -302,10 +304,10 @@ __device__ uint16_t* blk_hull(const Src& src, uint16_t* cur, uint16_t* nxt, uint
   return cur;
 }
 
-// From the sorted candidates m.b[0 .. m2) to the output, by the first T
-// threads of the CTA.
+// From the sorted candidates m.b[0 .. m2) to the hull (m.hn, m.hb), by the
+// first T threads of the CTA.
 template <int DT, int T, class M, class Src>
-__device__ void blk_tail(M& m, const Src& src, uint32_t m2, int32_t* out_idx, int32_t* out_count) {
+__device__ void blk_tail(M& m, const Src& src, uint32_t m2) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const BlkSet<DT>& s = m.s;
   // SPA: exclusive prefix minimum of the SPA value within each region,
@@ -360,13 +362,13 @@ __device__ void blk_tail(M& m, const Src& src, uint32_t m2, int32_t* out_idx, in
   uint32_t tot;
   uint32_t pre = blk_excl_sum<T>((uint32_t)__popc(keep), m.w32[0], tot);
   // the simple polygon: per region with E_r != E_{r+1}, E_r and the
-  // survivors in order; closed by the first point again
+  // survivors in order; closed by m.close (the first point again)
   const uint32_t flags = s.flags;
   uint32_t L = tot + 1;
 #pragma unroll
   for (int r = 0; r < 4; r++) L += !(flags & (SF_DEGEN0 << r));
   if (L == 1) {                               // every point identical
-    if (tid == 0) { out_idx[0] = src.out(s.eidx[0]); *out_count = 1; }
+    if (tid == 0) { m.a[0] = (uint16_t)s.eidx[0]; m.hn = 1; m.hb = 0; }
     return;
   }
   for (uint32_t i = i0; i < i1; i++) {
@@ -380,16 +382,14 @@ __device__ void blk_tail(M& m, const Src& src, uint32_t m2, int32_t* out_idx, in
   if (tid == 0) {
     const unsigned long long s2 = m.s2;       // complete: blk_excl_sum synchronised after the adds
     uint32_t o = 0;
-    int first = -1;
 #pragma unroll
     for (int r = 0; r < 4; r++) {
       if (!(flags & (SF_DEGEN0 << r))) {
         m.a[o++] = (uint16_t)(s.eidx[r] | kPin);
-        if (first < 0) first = r;
       }
       o += (uint32_t)(s2 >> (16 * r)) & 0xFFFFu;
     }
-    m.a[o] = (uint16_t)(s.eidx[first] | kPin);
+    m.a[o] = (uint16_t)(m.close | kPin);
   }
   blk_sync<T>();
   // identical neighbours: the first (smallest index) stays
@@ -409,8 +409,7 @@ __device__ void blk_tail(M& m, const Src& src, uint32_t m2, int32_t* out_idx, in
   blk_sync<T>();
   const bool flag = DT == DT_F64 ? (flags & SF_SMALL) != 0 : (flags & SF_WIDE) != 0;
   const uint16_t* h = blk_hull<DT, T>(src, m.b, m.a, reinterpret_cast<uint16_t*>(m.tab), m.dead, m.w32[0], m.w32[1], flag, L2);
-  for (uint32_t t = tid; t + 1 < L2; t += T) out_idx[t] = src.out(h[t] & ~kPin);
-  if (tid == 0) *out_count = (int32_t)(L2 - 1);
+  if (tid == 0) { m.hn = L2 - 1; m.hb = h == m.b; }
 }
 
 // Most sorted candidates that one warp takes to the end alone: it needs no
@@ -418,12 +417,13 @@ __device__ void blk_tail(M& m, const Src& src, uint32_t m2, int32_t* out_idx, in
 // other warps leave.
 constexpr uint32_t kBlkWarpTail = 256;
 
-// Steps 4-7 from the candidate list m.a[0 .. m.n[0]) to the output.  On entry
+// Steps 4-7 from the candidate list m.a[0 .. m.n[0]) to the hull (m.hn, m.hb;
+// not synchronised).  On entry
 // m.tab holds the smallest leading SPA word of the set's region-r points per
 // bucket (any subset of them), m.cnt and m.n[1..], m.s2 are zero, and the CTA
 // is synchronised.
 template <int DT, int CAP, int T, int NB, class Src>
-__device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src, int32_t* out_idx, int32_t* out_count) {
+__device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src) {
   using P = typename PT<DT>::T;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int Q = 4 * NB / T;               // buckets per thread
@@ -548,9 +548,9 @@ __device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src, int32_t* 
     __syncthreads();
   }
   if (m2 <= kBlkWarpTail) {
-    if (warp == 0) blk_tail<DT, 32>(m, src, m2, out_idx, out_count);
+    if (warp == 0) blk_tail<DT, 32>(m, src, m2);
   } else {
-    blk_tail<DT, T>(m, src, m2, out_idx, out_count);
+    blk_tail<DT, T>(m, src, m2);
   }
 }
 

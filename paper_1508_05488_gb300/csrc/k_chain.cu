@@ -133,6 +133,7 @@ constexpr size_t chain_local_smem() {
 
 template <int DT>
 __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   using P = typename PT<DT>::T;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
 
 template <int DT>
 __global__ void __launch_bounds__(kThreads) k_chain_merge(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   using P = typename PT<DT>::T;
   const int nseg = 4 * j.nsets;
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_merge(Job j, Ws w) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_output(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   __shared__ uint32_t sh_tile;
   __shared__ int sh_last;

@@ -274,6 +274,7 @@ __device__ __forceinline__ void oct_update(uint64_t dq[4], float X, float Y, uin
 
 template <int DT, bool OCT>
 __global__ void __launch_bounds__(kExtBlock, 2) k_extremes(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   using P = typename PointT<DT>::T;
   constexpr int PB = in_bytes<DT>();
@@ -723,6 +724,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_stairs(Job j, Ws w) {
   __shared__ float sqx[4], sqy[4];
   __shared__ int last;
   const int chunk = blockIdx.x;
+  if (sieved_leave(w)) return;
   int s = 0;
   if (j.sets) {
     int lo = 0, hi = j.nsets - 1;
@@ -1127,6 +1129,7 @@ __device__ __forceinline__ uint32_t a2_pass1_f32(const float* vx, const float* v
 // sub-slot) -- no block-wide barrier on the per-tile path.
 template <int DT, bool OCT>
 __global__ void __launch_bounds__(kClsBlock, 2) k_classify(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   using P = typename PointT<DT>::T;
   constexpr int PB = in_bytes<DT>();
@@ -1415,6 +1418,7 @@ __global__ void __launch_bounds__(kClsBlock, 2) k_classify(Job j, Ws w) {
 // most kSmallMax) and the multi-block sort, and plans both.
 
 __global__ void __launch_bounds__(kThreads) k_gather(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   constexpr int kChunkSub = kPlanTiles * kClsConsumers;     // sub-slots of a chunk
   static_assert(kChunkSub / kGatherSplitMax % kWarps == 0, "whole sub-slots per warp");

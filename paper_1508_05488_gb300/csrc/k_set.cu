@@ -15,6 +15,8 @@
 // The points are read four times by coalesced loads (extremes, the rescan of
 // the warps that hold one, regions, and the candidates); the set is at most
 // 256 KB, so every read after the first hits L1 or L2.
+#include <cooperative_groups.h>
+
 #include "hull_block.cuh"
 
 namespace cch {
@@ -34,26 +36,33 @@ template <>
 struct SetClass<3> { static constexpr int CAP = 16384, T = 512, NB = 1280; };
 static_assert(SetClass<kSetClasses - 1>::CAP == kSetMax + 1, "the largest class ends at kSetMax");
 
-struct SetSrcF64 {
+// Point c of the set, and the index it is reported as: its own, or that of the
+// sieve's list (`map`).
+template <int DT, bool LIST>
+struct SetSrc {
   const Job& j;
   int64_t off;
-  __device__ __forceinline__ double2 pt(uint32_t c) const { return input_point<double2>(j, off + c); }
-  __device__ __forceinline__ int32_t out(uint32_t c) const { return (int32_t)c; }
-};
-struct SetSrcI32 {
-  const Job& j;
-  int64_t off;
-  __device__ __forceinline__ int2 pt(uint32_t c) const { return input_point<int2>(j, off + c); }
-  __device__ __forceinline__ int32_t out(uint32_t c) const { return (int32_t)c; }
+  const uint32_t* map;
+  __device__ __forceinline__ typename PT<DT>::T pt(uint32_t c) const { return input_point<typename PT<DT>::T>(j, off + c); }
+  __device__ __forceinline__ int32_t out(uint32_t c) const { return LIST ? (int32_t)map[c] : (int32_t)c; }
 };
 
 // Order word of a leading word read as FP32, as a signed integer (-0.0 read as +0.0).
 __device__ __forceinline__ int32_t lead_order(float f) { return (int32_t)(f32_order(__fadd_rn(f, 0.0f)) ^ 0x80000000u); }
 
-// float32 vectors (DT_F64 with j.ys) are widened on load.
-template <int DT, int C>
-__global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* items) {
+// float32 vectors (DT_F64 with j.ys) are widened on load.  LIST: the points
+// that the sieve listed (j.pts), w.sv_hdr->n of them, by a cluster of four CTAs:
+// each does steps 1-3 on all points and steps 4-7 on one region, whose chain
+// ends in E1..E4, all of them vertices.  The listed points lie close to the
+// hull, so nearly all of them reach the last steps (2300 points of a 20M disk:
+// 57 us in one CTA, 45 of them from the sort on).
+template <int DT, int C, bool LIST>
+__global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* items, Ws w) {
   griddep_enter();
+  if (LIST) {
+    if (!sieved(w)) return;
+    griddep_release();                       // the pipeline has nothing to do (sieved_leave)
+  }
   constexpr int CAP = SetClass<C>::CAP, T = SetClass<C>::T, NB = SetClass<C>::NB, NW = T / 32;
   using P = typename PT<DT>::T;
   using M = BlkSmem<DT, CAP, T, NB>;
@@ -63,7 +72,8 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   __shared__ uint32_t red_amin[NW];
   __shared__ int32_t wext[4][NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const SetItem it = items ? items[blockIdx.x] : SetItem{0, (int32_t)j.N, 0};
+  const uint32_t part = LIST ? blockIdx.x : 0u;    // LIST: the CTA's region
+  const SetItem it = !LIST && items ? items[blockIdx.x] : SetItem{0, LIST ? (int32_t)w.sv_hdr->n : (int32_t)j.N, 0};
   const int n = it.n;
   int32_t* out_idx = j.out_idx + it.off;
   int32_t* out_count = j.out_counts + it.id;
@@ -71,7 +81,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
     if (tid == 0) *out_count = 0;
     return;
   }
-  typename std::conditional<DT == DT_F64, SetSrcF64, SetSrcI32>::type src{j, it.off};
+  const SetSrc<DT, LIST> src{j, it.off, w.cidx};
   for (int i = tid; i < 4 * NB; i += T) { m.tab[i] = 0xFFFFFFFFu; m.cnt[i] = 0u; }
   if (tid < 4) m.n[tid] = 0;
   if (tid == 0) m.s2 = 0;
@@ -241,7 +251,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   }
   __syncthreads();
   if (s.status != 0) {
-    if (tid == 0) *out_count = s.status;
+    if (tid == 0 && part == 0) *out_count = s.status;
     return;
   }
   // ---- steps 2-3: the first edge that has the point strictly outside is its
@@ -298,7 +308,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
       for (int u = 0; u < 4; u++) {
         const uint32_t i = (uint32_t)(i0 + u * T + tid), r = (rr >> (4 * u)) & 7u;
         e[u] = ((r - 1u) << 14) | i;
-        if (r != 0) {
+        if (LIST ? r == part + 1u : r != 0) {
           const P p = src.pt(i);
           atomicMin(&m.tab[(r - 1) * NB + blk_bucket<DT, NB>(s, p, (int)r - 1)],
                     blk_word<DT>(blk_spa<DT>(p, (int)r - 1)));
@@ -309,26 +319,64 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
     }
   }
   __syncthreads();
-  blk_finish<DT, CAP, T, NB>(m, src, out_idx, out_count);
+  uint32_t at = 0;                             // first output slot of the CTA's vertices
+  if constexpr (LIST) {
+    const uint32_t flags = s.flags, all = SF_DEGEN0 * 15u, mine = SF_DEGEN0 << part;
+    __syncthreads();
+    if (tid == 0) {
+      if ((flags & all) != all) s.flags = flags | (all & ~mine);   // this region's chain alone
+      m.close = s.eidx[(part + 1u) & 3u];
+      m.hn = 0;
+      m.hb = 0;
+    }
+    __syncthreads();
+    // a region between coincident extremes has no chain; all coincident: the
+    // first CTA's single point
+    if (!(flags & mine) || ((flags & all) == all && part == 0)) blk_finish<DT, CAP, T, NB>(m, src);
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    uint32_t tot = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < 4; q++) {
+      const uint32_t c = *cl.map_shared_rank(&m.hn, q);
+      at += q < part ? c : 0u;
+      tot += c;
+    }
+    cl.sync();                                 // nobody leaves while its count is read
+    if (tid == 0 && part == 0) *out_count = (int32_t)tot;
+  } else {
+    if (tid == 0) {
+      int k = 0;                               // the first region with a chain
+      while (k < 3 && (s.flags & (SF_DEGEN0 << k))) k++;
+      m.close = s.eidx[k];
+    }
+    blk_finish<DT, CAP, T, NB>(m, src);
+    __syncthreads();
+    if (tid == 0) *out_count = (int32_t)m.hn;
+  }
+  const uint16_t* h = m.hb ? m.b : m.a;
+  for (uint32_t t = tid; t < m.hn; t += T) out_idx[at + t] = src.out(h[t] & ~kPin);
 }
 
-template <int DT, int C>
-static void launch_set_c(const Job& j, const SetItem* items, int count, cudaStream_t st) {
+template <int DT, int C, bool LIST>
+static void launch_set_c(const Job& j, const SetItem* items, const Ws& w, int count, cudaStream_t st) {
   constexpr size_t sm = sizeof(BlkSmem<DT, SetClass<C>::CAP, SetClass<C>::T, SetClass<C>::NB>);
   static bool once = [] {
-    cudaFuncSetAttribute(k_set<DT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_set<DT, C, LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     return true;
   }();
   (void)once;
-  launch_pdl(k_set<DT, C>, count, SetClass<C>::T, sm, st, j, items);
+  if (LIST) launch_pdl_cluster(k_set<DT, C, LIST>, 4, SetClass<C>::T, 4, sm, st, j, items, w);
+  else launch_pdl(k_set<DT, C, LIST>, count, SetClass<C>::T, sm, st, j, items, w);
 }
 
 template <int DT>
 static void launch_set_t(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st) {
-  if (cls == 0) launch_set_c<DT, 0>(j, items, count, st);
-  else if (cls == 1) launch_set_c<DT, 1>(j, items, count, st);
-  else if (cls == 2) launch_set_c<DT, 2>(j, items, count, st);
-  else launch_set_c<DT, 3>(j, items, count, st);
+  if (cls == 0) launch_set_c<DT, 0, false>(j, items, Ws{}, count, st);
+  else if (cls == 1) launch_set_c<DT, 1, false>(j, items, Ws{}, count, st);
+  else if (cls == 2) launch_set_c<DT, 2, false>(j, items, Ws{}, count, st);
+  else launch_set_c<DT, 3, false>(j, items, Ws{}, count, st);
 }
 
 int set_class(int64_t n) {
@@ -339,6 +387,15 @@ int launch_set(const Job& j, int cls, const SetItem* items, int count, cudaStrea
   if (count == 0) return 0;
   if (j.dtype == DT_I32) launch_set_t<DT_I32>(j, cls, items, count, st);
   else launch_set_t<DT_F64>(j, cls, items, count, st);
+  return 1;
+}
+
+int launch_set_list(const Job& j, const Ws& w, cudaStream_t st) {
+  Job l = j;
+  l.pts = w.cpts;          // float32 vectors are listed widened
+  l.ys = nullptr;
+  if (j.dtype == DT_I32) launch_set_c<DT_I32, 3, true>(l, nullptr, w, 1, st);
+  else launch_set_c<DT_F64, 3, true>(l, nullptr, w, 1, st);
   return 1;
 }
 

@@ -231,6 +231,7 @@ __device__ __forceinline__ void prefix_min_excl(uint32_t* t, uint32_t seed, uint
 
 template <int DT, int CL>
 __global__ void __launch_bounds__(kSmThreads, 1) k_small(Job j, Ws w) {
+  if (sieved_leave(w)) return;
   griddep_enter();
   namespace cg = cooperative_groups;
   using P = typename std::conditional<DT == DT_F64, double2, int2>::type;
