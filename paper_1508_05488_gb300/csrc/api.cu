@@ -83,9 +83,9 @@ Layout layout(const Dims& d, char* base) {
   L.w.blk_tail = (int32_t*)take(4 * (size_t)d.max_chain_blks);
   L.w.out_start = (uint32_t*)take(4 * (4 * (size_t)d.nsets + 1));
   L.w.stairs = (uint32_t*)take(4 * 4 * (size_t)kStairB * d.nsets);
-  L.w.sv_hdr = (SieveHdr*)take(sizeof(SieveHdr));
-  L.w.sv_tab = (float4*)take(sieve_table_bytes());
-  L.w.sv_cnt = (uint32_t*)take(4 * (size_t)kSvMaxUnits);
+  L.w.sv_hdr = (SieveHdr*)take(sizeof(SieveHdr) * d.nsets);
+  L.w.sv_tab = (float4*)take(2 * sizeof(float4) * std::max<size_t>(kSvRows + 2, (size_t)(kSvBatchRows + 2) * d.nsets));
+  L.w.sv_cnt = (uint32_t*)take(4 * std::max<size_t>(kSvMaxUnits, kSvWarps * ((size_t)d.N / (kSvWarps * kSvBatchLen) + d.nsets + 1)));
   L.total = o;
   return L;
 }
@@ -185,17 +185,21 @@ struct StageOut {
 // The sets of a batch: the pipeline's, and the small ones of k_set by class.
 struct Batch {
   std::vector<SetDesc> sets;
+  std::vector<SieveSet> sieve;           // of the pipeline's sets
+  std::vector<int32_t> cta;              // set of every k_sieve CTA
   std::vector<SetItem> items[kSetClasses];
 };
 
-// Copy a batch's tables (small sets by class, then the pipeline's sets) to the
+// Copy a batch's tables (small sets by class, then the larger sets) to the
 // device, and launch k_set on the small ones.  Called with g_mu held; returns
 // a status, the kernels launched are added to *nk.
 int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int* nk) {
   size_t ibytes = 0;
   for (const auto& v : b.items) ibytes += sizeof(SetItem) * v.size();
   const size_t sets_off = (ibytes + 63) / 64 * 64;
-  const size_t bytes = sets_off + sizeof(SetDesc) * b.sets.size();
+  const size_t sv_off = sets_off + (sizeof(SetDesc) * b.sets.size() + 63) / 64 * 64;
+  const size_t cta_off = sv_off + sizeof(SieveSet) * b.sieve.size();
+  const size_t bytes = cta_off + sizeof(int32_t) * b.cta.size();
   if (!ws->tab_done && cudaEventCreateWithFlags(&ws->tab_done, cudaEventDisableTiming) != cudaSuccess) return CCH_ERR_CUDA;
   if (cudaEventSynchronize(ws->tab_done) != cudaSuccess) return CCH_ERR_CUDA;
   if (ws->tab_bytes < bytes) {
@@ -218,15 +222,32 @@ int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int*
     if (!v.empty()) memcpy(ws->host_tab + o, v.data(), sizeof(SetItem) * v.size());
     o += sizeof(SetItem) * v.size();
   }
-  if (!b.sets.empty()) memcpy(ws->host_tab + sets_off, b.sets.data(), sizeof(SetDesc) * b.sets.size());
+  if (!b.sets.empty()) {
+    memcpy(ws->host_tab + sets_off, b.sets.data(), sizeof(SetDesc) * b.sets.size());
+    memcpy(ws->host_tab + sv_off, b.sieve.data(), sizeof(SieveSet) * b.sieve.size());
+    if (!b.cta.empty()) memcpy(ws->host_tab + cta_off, b.cta.data(), sizeof(int32_t) * b.cta.size());
+  }
   if (cudaMemcpyAsync(ws->dev_tab, ws->host_tab, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
   if (cudaEventRecord(ws->tab_done, stream) != cudaSuccess) return CCH_ERR_CUDA;
   const SetItem* items = reinterpret_cast<const SetItem*>(ws->dev_tab);
   o = 0;
   for (int c = 0; c < kSetClasses; c++) o += b.items[c].size();
-  for (int c = kSetClasses - 1; c >= 0; c--) {     // the largest sets first
+  // the largest sets first; a class starts beside the one before it where that
+  // leaves SMs free (1024 int32 sets, 213, 103, 94 and 205 of them small: 285 us
+  // a call, 343 one class after the other); where it does not, sharing an SM
+  // costs both their L1 (4096 float64 sets of 256 to 4096 points: 259 us
+  // beside, 224 one after the other)
+  size_t prev = 0;
+  for (int c = kSetClasses - 1; c >= 0; c--) {
     o -= b.items[c].size();
-    *nk += launch_set(j, c, items + o, (int)b.items[c].size(), stream);
+    const bool beside = prev != 0 && prev <= 2 * (size_t)sm_count();
+    if (!b.items[c].empty()) prev = b.items[c].size();
+    *nk += launch_set(j, c, items + o, (int)b.items[c].size(), beside, stream);
+  }
+  if (!b.cta.empty()) {
+    j.sv_sets = reinterpret_cast<const SieveSet*>(ws->dev_tab + sv_off);
+    j.sv_cta = reinterpret_cast<const int32_t*>(ws->dev_tab + cta_off);
+    j.sv_nctas = (int32_t)b.cta.size();
   }
   j.sets = reinterpret_cast<const SetDesc*>(ws->dev_tab + sets_off);
   return CCH_OK;
@@ -267,7 +288,7 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   auto mark = [&](int k) {
     if (ev && ((rec.mask >> k) & 1u || (k > 0 && (rec.mask >> (k - 1)) & 1u))) cudaEventRecord(ev[k], stream);
   };
-  if (j.sieve.nunit) nk += launch_sieve(j, L.w, stream);
+  if (j.sieve.nunit || j.sv_sets) nk += launch_sieve(j, L.w, stream);
   mark(0);
   nk += launch_extremes(j, L.w, La);
   mark(1);
@@ -346,7 +367,7 @@ Job set_job(const void* points, const float* ys, int64_t n, int dtype, int32_t* 
 }
 
 int run_set(const Job& j, cudaStream_t stream) {
-  g_launches += (uint64_t)launch_set(j, set_class(j.N), nullptr, 1, stream);
+  g_launches += (uint64_t)launch_set(j, set_class(j.N), nullptr, 1, false, stream);
   return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
 }
 
@@ -417,6 +438,9 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
     int32_t cp = (t + kPlanTiles - 1) / kPlanTiles;
     batch.sets.push_back(
         SetDesc{offsets[s], n, (int32_t)nch, c, (int32_t)nt, t, (int32_t)n3, c3, (int32_t)np_, cp, s});
+    const SieveSet sv = sieve_batch_set(offsets[s], n, (int32_t)batch.cta.size());
+    batch.cta.insert(batch.cta.end(), (size_t)(sv.nunit + kSvWarps - 1) / kSvWarps, (int32_t)batch.sieve.size());
+    batch.sieve.push_back(sv);
     nch += c;
     nt += t;
     n3 += c3;

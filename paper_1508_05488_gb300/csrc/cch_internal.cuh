@@ -38,6 +38,7 @@ enum : int {
   ST_NOMEM = -5,
   ST_CUDA = -6,
   ST_TIMEOUT = -7,
+  ST_SIEVED = 1,        // not an error: a batch's set that the sieve has finished
 };
 
 // Input formats.  DT_F32 (two float32 coordinate vectors) is read by the
@@ -136,6 +137,7 @@ enum : int {
   CT_SPA_TOTAL,
   CT_CHAIN_TOTAL,
   CT_OUT_TOTAL,
+  CT_SIEVE_SETS,                       // sets of a batch finished by the sieve path
   CT_SIEVED,                           // the set was finished by the sieve path: the pipeline's kernels leave
   CT_ERR,                              // first device error (negative status)
   CT_COUNT
@@ -180,8 +182,15 @@ struct SieveSet {
   int64_t len;          // points per unit
   int32_t nunit;
   int32_t pre;          // points at the head of every unit that are prefetched
+  int32_t cta0;         // first k_sieve CTA (kSvWarps units each)
+  int32_t pad;
 };
-constexpr int kSvMaxUnits = 5120;
+constexpr int kSvMaxUnits = 5120;      // of a single set
+constexpr int kSvWarps = 8;            // warps, hence units, per k_sieve CTA
+// A batch's larger sets: units of kSvBatchLen points, kSvBatchUnits per set at
+// most (larger sets take the pipeline), tables of kSvBatchRows bands.
+constexpr int kSvBatchLen = 2048, kSvBatchUnits = 1024, kSvBatchRows = 256;
+constexpr int kSvRows = 512;           // bands per axis of a single set's table
 // Device side of it: the maps of the bands (of Y: s[0] Y + o[0], of X: s[1] X +
 // o[1]), whether the sieve runs (mode) and the number of listed points.
 struct alignas(16) SieveHdr {
@@ -207,7 +216,10 @@ struct Job {
   Tune tune;            // run-time choices (the same results with any valid choice)
   const SetDesc* sets;  // device array, or nullptr -> use `one`
   SetDesc one;
-  SieveSet sieve;       // nunit 0: the call does not sieve
+  SieveSet sieve;       // a single set (nunit 0: the call does not sieve it)
+  const SieveSet* sv_sets;   // a batch: device array beside `sets`, nullptr: no sieve
+  const int32_t* sv_cta;     // a batch: set of every k_sieve CTA
+  int32_t sv_nctas;
   int32_t* out_idx;     // device
   int32_t* out_counts;  // device, [nsets]
   int32_t* r1_idx;      // stage hook (set 0, or nullptr): round-1 survivors, region-major
@@ -300,6 +312,7 @@ struct Ws {
   SieveHdr* sv_hdr;          // the sieve's header, band table and listed points per unit
   float4* sv_tab;
   uint32_t* sv_cnt;
+  const void* sv_in;         // k_set on lists: the call's points
 };
 
 // Chain slots of (set s, region r) when the region's records start at `rbase`
@@ -1018,10 +1031,10 @@ struct Launch {
 
 // Each returns the number of kernels it launched.
 int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
-int launch_set(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st);   // items null: the one set
+int launch_set(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st);   // items null: the one set
 int launch_set_list(const Job& j, const Ws& w, cudaStream_t st);   // the sieve's listed points
 SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);
-size_t sieve_table_bytes();
+SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0);
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st);
 int launch_extremes(const Job& j, const Ws& w, const Launch& L);
 int launch_stairs(const Job& j, const Ws& w, const Launch& L);

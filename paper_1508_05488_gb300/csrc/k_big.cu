@@ -125,7 +125,7 @@ __device__ void plan_chain(const Job& j, const Ws& w) {
       const SetCtl& c = w.ctl[s];
       const uint32_t degen_all = (SF_DEGEN0 * 15u);
       if (c.status != 0) {
-        if (r == 0) j.out_counts[sd.id] = c.status;
+        if (r == 0 && c.status < 0) j.out_counts[sd.id] = c.status;
       } else if (sd.n == 0) {
         if (r == 0) j.out_counts[sd.id] = 0;
       } else if ((c.flags & degen_all) == degen_all) {

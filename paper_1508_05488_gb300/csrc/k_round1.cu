@@ -302,6 +302,7 @@ __global__ void __launch_bounds__(kExtBlock, 2) k_extremes(Job j, Ws w) {
     }
     s = lo;
   }
+  if (j.sv_sets && w.ctl[s].status == ST_SIEVED) return;   // uniform
   const SetDesc sd = get_set(j, s);
   const int64_t tiles_set = (sd.n + TILE - 1) / TILE;
   const int64_t k0 = chunk - sd.chunk1, kstep = sd.nchunk1;
@@ -734,7 +735,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_stairs(Job j, Ws w) {
     }
     s = lo;
   }
-  if (j.opts & OPT_NO_PREFILTER) {   // uniform; the table is unused
+  // (a sieved set's status was written before a1's wait ended)
+  if ((j.opts & OPT_NO_PREFILTER) || (j.sv_sets && *(volatile int32_t*)&w.ctl[s].status == ST_SIEVED)) {   // uniform; the table is unused
     griddep_enter();   // every CTA exits after a1 has completed: a2 waits for k_stairs only
     return;
   }

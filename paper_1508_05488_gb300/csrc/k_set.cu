@@ -50,19 +50,29 @@ struct SetSrc {
 // Order word of a leading word read as FP32, as a signed integer (-0.0 read as +0.0).
 __device__ __forceinline__ int32_t lead_order(float f) { return (int32_t)(f32_order(__fadd_rn(f, 0.0f)) ^ 0x80000000u); }
 
-// float32 vectors (DT_F64 with j.ys) are widened on load.  LIST: the points
-// that the sieve listed (j.pts), w.sv_hdr->n of them, by a cluster of four CTAs:
+// What k_set works on: the points of whole sets (items, or the one set); a
+// single set's list from the sieve, w.sv_hdr->n points; or the lists of a
+// batch's larger sets, which each CTA first gathers from its set's units.
+enum : int { SET_WHOLE = 0, SET_LIST = 1, SET_BATCH = 2 };
+
+// float32 vectors (DT_F64 with j.ys) are widened on load.  `beside`: the kernel
+// before this one works on other sets of the same call, so this one starts
+// beside it, and one of its CTAs waits for its end (all of them waiting would
+// hold the SMs: 4096 small float64 sets 246 us, 220 without the overlap).
+// SET_LIST: the listed points (j.pts) are finished by a cluster of four CTAs:
 // each does steps 1-3 on all points and steps 4-7 on one region, whose chain
 // ends in E1..E4, all of them vertices.  The listed points lie close to the
 // hull, so nearly all of them reach the last steps (2300 points of a 20M disk:
 // 57 us in one CTA, 45 of them from the sort on).
-template <int DT, int C, bool LIST>
-__global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* items, Ws w) {
-  griddep_enter();
-  if (LIST) {
+template <int DT, int C, int MODE>
+__global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* items, Ws w, bool beside) {
+  constexpr bool LIST = MODE == SET_LIST;
+  if (MODE != SET_WHOLE || !beside) griddep_enter();
+  if constexpr (LIST) {
     if (!sieved(w)) return;
     griddep_release();                       // the pipeline has nothing to do (sieved_leave)
   }
+  if constexpr (MODE == SET_WHOLE) griddep_release();
   constexpr int CAP = SetClass<C>::CAP, T = SetClass<C>::T, NB = SetClass<C>::NB, NW = T / 32;
   using P = typename PT<DT>::T;
   using M = BlkSmem<DT, CAP, T, NB>;
@@ -73,15 +83,51 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   __shared__ int32_t wext[4][NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t part = LIST ? blockIdx.x : 0u;    // LIST: the CTA's region
-  const SetItem it = !LIST && items ? items[blockIdx.x] : SetItem{0, LIST ? (int32_t)w.sv_hdr->n : (int32_t)j.N, 0};
+  SetItem it = MODE == SET_WHOLE && items ? items[blockIdx.x] : SetItem{0, LIST ? (int32_t)w.sv_hdr->n : (int32_t)j.N, 0};
+  if constexpr (MODE == SET_BATCH) {
+    // gather the set's list; a list of another size class, or too long a one
+    // (the pipeline's), is left
+    const SieveSet sv = j.sv_sets[blockIdx.x];
+    if (w.sv_hdr[blockIdx.x].mode == 0) return;
+    const uint32_t* cnt = w.sv_cnt + (size_t)sv.cta0 * kSvWarps;
+    static_assert(kSvBatchUnits <= 4 * NB && kSvBatchUnits % T == 0, "the units' prefix fits the table");
+    constexpr int PU = kSvBatchUnits / T;
+    uint32_t c[PU], sum = 0, total;
+#pragma unroll
+    for (int q = 0; q < PU; q++) { const int u = tid * PU + q; c[q] = u < sv.nunit ? cnt[u] : 0u; sum += c[q]; }
+    uint32_t pre = blk_excl_sum<T>(sum, m.w32[0], total);
+    if (total > (uint32_t)kSetMax || (total < (uint32_t)SetClass<2>::CAP) != (C == 2)) return;
+#pragma unroll
+    for (int q = 0; q < PU; q++) { m.tab[tid * PU + q] = pre; pre += c[q]; }
+    __syncthreads();
+    P* lp = reinterpret_cast<P*>(w.cpts) + sv.off;       // j.pts is w.cpts
+    const P* in = reinterpret_cast<const P*>(w.sv_in) + sv.off;
+    for (uint32_t p = tid; p < total; p += T) {
+      uint32_t l = 0, h = kSvBatchUnits - 1;             // the last unit that starts at or before p
+      while (l < h) {
+        const uint32_t q = (l + h + 1) >> 1;
+        if (m.tab[q] <= p) l = q; else h = q - 1;
+      }
+      const uint32_t g = w.valA[sv.off + (int64_t)l * sv.len + (p - m.tab[l])];
+      lp[p] = in[g];
+      w.cidx[sv.off + p] = g;
+    }
+    __syncthreads();
+    it = SetItem{sv.off, (int32_t)total, j.sets[blockIdx.x].id};
+    if (tid == 0) {
+      w.ctl[blockIdx.x].status = ST_SIEVED;
+      if (atomicAdd(w.ctr + CT_SIEVE_SETS, 1u) + 1u == (uint32_t)j.nsets) w.ctr[CT_SIEVED] = 1u;
+    }
+  }
   const int n = it.n;
   int32_t* out_idx = j.out_idx + it.off;
   int32_t* out_count = j.out_counts + it.id;
   if (n == 0) {
     if (tid == 0) *out_count = 0;
+    if (MODE == SET_WHOLE && beside && blockIdx.x == 0) griddep_enter();
     return;
   }
-  const SetSrc<DT, LIST> src{j, it.off, w.cidx};
+  const SetSrc<DT, MODE != SET_WHOLE> src{j, it.off, MODE == SET_BATCH ? w.cidx + it.off : w.cidx};
   for (int i = tid; i < 4 * NB; i += T) { m.tab[i] = 0xFFFFFFFFu; m.cnt[i] = 0u; }
   if (tid < 4) m.n[tid] = 0;
   if (tid == 0) m.s2 = 0;
@@ -252,6 +298,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   __syncthreads();
   if (s.status != 0) {
     if (tid == 0 && part == 0) *out_count = s.status;
+    if (MODE == SET_WHOLE && beside && blockIdx.x == 0) griddep_enter();
     return;
   }
   // ---- steps 2-3: the first edge that has the point strictly outside is its
@@ -357,46 +404,57 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   }
   const uint16_t* h = m.hb ? m.b : m.a;
   for (uint32_t t = tid; t < m.hn; t += T) out_idx[at + t] = src.out(h[t] & ~kPin);
+  if (MODE == SET_WHOLE && beside && blockIdx.x == 0) griddep_enter();
 }
 
-template <int DT, int C, bool LIST>
-static void launch_set_c(const Job& j, const SetItem* items, const Ws& w, int count, cudaStream_t st) {
+template <int DT, int C, int MODE>
+static void launch_set_c(const Job& j, const SetItem* items, const Ws& w, int count, bool beside, cudaStream_t st) {
   constexpr size_t sm = sizeof(BlkSmem<DT, SetClass<C>::CAP, SetClass<C>::T, SetClass<C>::NB>);
   static bool once = [] {
-    cudaFuncSetAttribute(k_set<DT, C, LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_set<DT, C, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     return true;
   }();
   (void)once;
-  if (LIST) launch_pdl_cluster(k_set<DT, C, LIST>, 4, SetClass<C>::T, 4, sm, st, j, items, w);
-  else launch_pdl(k_set<DT, C, LIST>, count, SetClass<C>::T, sm, st, j, items, w);
+  launch_pdl_cluster(k_set<DT, C, MODE>, count, SetClass<C>::T, MODE == SET_LIST ? 4 : 1, sm, st, j, items, w, beside);
 }
 
 template <int DT>
-static void launch_set_t(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st) {
-  if (cls == 0) launch_set_c<DT, 0, false>(j, items, Ws{}, count, st);
-  else if (cls == 1) launch_set_c<DT, 1, false>(j, items, Ws{}, count, st);
-  else if (cls == 2) launch_set_c<DT, 2, false>(j, items, Ws{}, count, st);
-  else launch_set_c<DT, 3, false>(j, items, Ws{}, count, st);
+static void launch_set_t(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st) {
+  if (cls == 0) launch_set_c<DT, 0, SET_WHOLE>(j, items, Ws{}, count, beside, st);
+  else if (cls == 1) launch_set_c<DT, 1, SET_WHOLE>(j, items, Ws{}, count, beside, st);
+  else if (cls == 2) launch_set_c<DT, 2, SET_WHOLE>(j, items, Ws{}, count, beside, st);
+  else launch_set_c<DT, 3, SET_WHOLE>(j, items, Ws{}, count, beside, st);
 }
 
 int set_class(int64_t n) {
   return n < SetClass<0>::CAP ? 0 : n < SetClass<1>::CAP ? 1 : n < SetClass<2>::CAP ? 2 : n <= kSetMax ? 3 : -1;
 }
 
-int launch_set(const Job& j, int cls, const SetItem* items, int count, cudaStream_t st) {
+int launch_set(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st) {
   if (count == 0) return 0;
-  if (j.dtype == DT_I32) launch_set_t<DT_I32>(j, cls, items, count, st);
-  else launch_set_t<DT_F64>(j, cls, items, count, st);
+  if (j.dtype == DT_I32) launch_set_t<DT_I32>(j, cls, items, count, beside, st);
+  else launch_set_t<DT_F64>(j, cls, items, count, beside, st);
   return 1;
+}
+
+template <int DT>
+static int launch_set_list_t(const Job& l, const Ws& w, cudaStream_t st) {
+  if (!l.sv_sets) {
+    launch_set_c<DT, 3, SET_LIST>(l, nullptr, w, 4, false, st);
+    return 1;
+  }
+  launch_set_c<DT, 2, SET_BATCH>(l, nullptr, w, l.nsets, false, st);
+  launch_set_c<DT, 3, SET_BATCH>(l, nullptr, w, l.nsets, false, st);
+  return 2;
 }
 
 int launch_set_list(const Job& j, const Ws& w, cudaStream_t st) {
   Job l = j;
   l.pts = w.cpts;          // float32 vectors are listed widened
   l.ys = nullptr;
-  if (j.dtype == DT_I32) launch_set_c<DT_I32, 3, true>(l, nullptr, w, 1, st);
-  else launch_set_c<DT_F64, 3, true>(l, nullptr, w, 1, st);
-  return 1;
+  Ws v = w;
+  v.sv_in = j.pts;
+  return j.dtype == DT_I32 ? launch_set_list_t<DT_I32>(l, v, st) : launch_set_list_t<DT_F64>(l, v, st);
 }
 
 }  // namespace cch

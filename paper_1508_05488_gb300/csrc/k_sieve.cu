@@ -14,6 +14,8 @@
 //              many it builds the polygon of the listed points themselves and
 //              lists only those outside it;
 //   k_set      (k_set.cu) runs the method (Sec. 2.1) on the listed points.
+// A batch's sets above kSetMax points go the same way, every set with a table
+// of its own (one CTA) and without k_refine.
 // Sets whose points mostly lie on or beside their hull (the sample tells) take
 // the pipeline, which k_refine's flag lets the later launches know.
 //
@@ -50,8 +52,8 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int kTabThreads = 1024;
-constexpr int kTabWarps = kTabThreads / 32;
+constexpr int kTabThreads = 1024;                   // of k_refine, and of k_table on a single set
+constexpr int kTabBatchThreads = 512;               // of k_table on a batch's sets
 constexpr int kTabItems = 8;                        // sample points per thread at most
 constexpr int kPeel = 40;                           // peeling rounds at most
 constexpr uint32_t kPlain = 2048;                   // lists up to this size go to k_set as they are
@@ -104,18 +106,19 @@ __device__ __forceinline__ bool sieve_inside(const float4* tab, const SieveHdr& 
 
 // Sides: 0 left, 1 right (bands u = Y, compared v = X, -X), 2 bottom, 3 top
 // (u = X, v = Y, -Y).  A polyline point is (v, u).
-template <int R>
+template <int R, int T>
 struct TabSmem {
+  static constexpr int W = T / 32;
   uint2 bv[2][R];               // per axis and band: order words of the smallest v of its two sides
   uint2 bu[2][R];               // bits of those points' u
   float2 pl[4][2][R + 2];       // polylines, ping-pong
-  uint64_t ext[kTabWarps][4];
+  uint64_t ext[W][4];
   uint64_t gext[4];             // this CTA's extremes, read by the cluster
-  uint32_t w32[4][2][kTabWarps / 4];
+  uint32_t w32[4][2][W / 4];
   uint32_t plen[4], pbuf[4];    // the polylines' lengths and buffers
   uint32_t cnt;                 // leader: sample points outside; k_refine: points kept
-  uint32_t pre[kTabWarps];
-  uint32_t upre[kSvMaxUnits];   // k_refine: listed points before each unit
+  uint32_t pre[W];
+  uint32_t upre[T == kTabThreads ? kSvMaxUnits : 1];   // k_refine: listed points before each unit
 };
 
 __device__ __forceinline__ float unorder(uint32_t k) {
@@ -134,8 +137,9 @@ __device__ __forceinline__ T* cl_map(T* p, int r) {
 }
 
 // Barrier of one side's quarter of the CTA.
+template <int T>
 __device__ __forceinline__ void side_sync(int side) {
-  asm volatile("bar.sync %0, %1;" :: "r"(side + 1), "r"(kTabThreads / 4) : "memory");
+  asm volatile("bar.sync %0, %1;" :: "r"(side + 1), "r"(T / 4) : "memory");
 }
 
 // Inclusive warp prefix sum.
@@ -153,8 +157,8 @@ __device__ __forceinline__ uint32_t warp_incl_sum(uint32_t x) {
 // bit k: item k), by every thread of the cluster.  They go to `tab` and `hdr`
 // (global memory) and are visible to the cluster on return; false where there
 // are none.
-template <int R, int CL>
-__device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const float (&Y)[kTabItems], uint32_t valid,
+template <int R, int CL, int T>
+__device__ bool build_table(TabSmem<R, T>& m, const float (&X)[kTabItems], const float (&Y)[kTabItems], uint32_t valid,
                             int rank, float4* tab, SieveHdr* hdr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // extremes: per side the smallest v (and the smallest u among them)
@@ -175,10 +179,10 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
       e[q] = u64_warp_min(e[q]);
       if (lane == 0) m.ext[warp][q] = e[q];
     }
-    for (int i = tid; i < 2 * R; i += kTabThreads) (&m.bv[0][0])[i] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+    for (int i = tid; i < 2 * R; i += T) (&m.bv[0][0])[i] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
     __syncthreads();
     if (warp < 4) {
-      const uint64_t g = u64_warp_min(m.ext[lane][warp]);
+      const uint64_t g = u64_warp_min(lane < T / 32 ? m.ext[lane][warp] : ~0ull);
       if (lane == 0) m.gext[warp] = g;
     }
     if (tid == 0) m.cnt = 0;
@@ -239,7 +243,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
   if constexpr (CL > 1) {
     // each CTA merges its share of the bands into the leader's copy
     constexpr int S = 4 * R / CL;                    // words
-    static_assert(S <= kTabThreads, "one band word per thread");
+    static_assert(S <= T, "one band word per thread");
     if (tid < S) {
       const int i = rank * S + tid;
       uint32_t w[CL], v[CL];
@@ -260,7 +264,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
   }
   if (rank == 0) {
     // one side per quarter of the CTA: polyline of the band points, then peeling
-    constexpr int H = kTabThreads / 4, HW = H / 32, PB = (R + H - 1) / H, Q = (R + 2 + H - 1) / H;
+    constexpr int H = T / 4, HW = H / 32, PB = (R + H - 1) / H, Q = (R + 2 + H - 1) / H;
     const int side = tid / H, t = tid - side * H, sw = t >> 5;
     float2* cur = m.pl[side][0];
     float2* nxt = m.pl[side][1];
@@ -275,7 +279,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
       for (int q = 0; q < PB; q++) { const int b = t * PB + q; c += b < R && bv[2 * b] != 0xFFFFFFFFu; }
       const uint32_t x = warp_incl_sum(c);
       if (lane == 31) m.w32[side][0][sw] = x;
-      side_sync(side);
+      side_sync<T>(side);
       uint32_t pre = x - c + 1, tot = 0;
 #pragma unroll
       for (int q = 0; q < HW; q++) { const uint32_t v = m.w32[side][0][q]; pre += q < sw ? v : 0u; tot += v; }
@@ -292,7 +296,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
       const uint64_t elo = side < 2 ? e[2] : e[0], ehi = side < 2 ? e[3] : e[1];
       if (t == 0) cur[0] = make_float2(unorder((uint32_t)elo), unorder((uint32_t)(elo >> 32)));
       if (t == 1) cur[n - 1] = make_float2(unorder((uint32_t)ehi), unorder(~(uint32_t)(ehi >> 32)));
-      side_sync(side);
+      side_sync<T>(side);
     }
     auto keeps = [&](uint32_t i) {
       if (i == 0 || i == n - 1) return true;
@@ -311,7 +315,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
       const uint32_t c = __popc(keep), x = warp_incl_sum(c);
       uint32_t* sh = m.w32[side][(round + 1) & 1];
       if (lane == 31) sh[sw] = x;
-      side_sync(side);
+      side_sync<T>(side);
       uint32_t pre = x - c, tot = 0;
 #pragma unroll
       for (int q = 0; q < HW; q++) { const uint32_t v = sh[q]; pre += q < sw ? v : 0u; tot += v; }
@@ -322,7 +326,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
           if ((keep >> q) & 1u) nxt[pre++] = cur[i0 + q];
         float2* z = cur; cur = nxt; nxt = z;
         n = tot;
-        side_sync(side);
+        side_sync<T>(side);
       }
     }
     // the rest by the side's first warp, without CTA barriers
@@ -360,7 +364,7 @@ __device__ bool build_table(TabSmem<R>& m, const float (&X)[kTabItems], const fl
       return __fmaf_rn(f, b.x - a.x, a.x);
     };
     const float inf = __int_as_float(0x7F800000);
-    for (int i = tid; i < 2 * R + 4; i += kTabThreads) {
+    for (int i = tid; i < 2 * R + 4; i += T) {
       const int ax = i < 2 * R ? i / R : i & 1;                  // the 2 R bands, then the four ends
       const int b = i < 2 * R ? i - ax * R + 1 : (i - 2 * R) / 2 * (R + 1);
       const float u0 = ax ? x0 : y0, u1 = ax ? x1 : y1, um = ax ? xm : ym, vm = ax ? ym : xm;
@@ -397,30 +401,36 @@ __device__ __forceinline__ SieveHdr fresh_hdr(const SieveHdr* h) {
 }
 
 // Table of each set from a sample spread over it in runs of 32 points.
-template <int DT, int R, int CL>
-__global__ void __launch_bounds__(kTabThreads, 1) k_table(Job j, Ws w) {
+template <int DT, int R, int CL, int T>
+__global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   griddep_enter();
   extern __shared__ __align__(16) unsigned char smem[];
-  TabSmem<R>& m = *reinterpret_cast<TabSmem<R>*>(smem);
+  TabSmem<R, T>& m = *reinterpret_cast<TabSmem<R, T>*>(smem);
+  constexpr int W = T / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = blockIdx.x % CL;
-  const SieveSet sd = j.sieve;
-  SieveHdr* hdr = w.sv_hdr;
-  float4* tab = w.sv_tab;
+  const int set = blockIdx.x / CL;
+  const SieveSet sd = j.sv_sets ? j.sv_sets[set] : j.sieve;
+  SieveHdr* hdr = w.sv_hdr + set;
+  float4* tab = w.sv_tab + (size_t)set * 2 * (R + 2);
+  if (sd.nunit == 0) {                                 // uniform over the cluster
+    if (rank == 0 && tid == 0) hdr->mode = 0;
+    return;
+  }
   // at most n / 8 points in runs of 32
-  const int64_t groups = min((int64_t)CL * kTabWarps * kTabItems, max(sd.n / 256, (int64_t)1));
+  const int64_t groups = min((int64_t)CL * W * kTabItems, max(sd.n / 256, (int64_t)1));
   const int64_t step = sd.n / groups;
   float X[kTabItems], Y[kTabItems];
   uint32_t valid = 0;
 #pragma unroll
   for (int k = 0; k < kTabItems; k++) {
-    const int64_t g = ((int64_t)k * CL + rank) * kTabWarps + warp;
+    const int64_t g = ((int64_t)k * CL + rank) * W + warp;
     X[k] = Y[k] = 0.f;
     if (g < groups) valid |= (uint32_t)sieve_view<DT>(j, sd.off + g * step + lane, X[k], Y[k]) << k;
   }
   // the sample is here: k_sieve's CTAs may start and prefetch
   griddep_release();
-  const bool ok = build_table<R, CL>(m, X, Y, valid, rank, tab, hdr);
+  const bool ok = build_table<R, CL, T>(m, X, Y, valid, rank, tab, hdr);
   // what is left of the first item of every thread tells whether the sieve pays
   uint32_t outn = 0;
   if (ok) {
@@ -431,13 +441,12 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_table(Job j, Ws w) {
     cl_sync<CL>();
   }
   if (rank == 0 && tid == 0) {
-    const int64_t left = ok ? (int64_t)m.cnt * sd.n / (min(groups, (int64_t)CL * kTabWarps) * 32) : sd.n;
+    const int64_t left = ok ? (int64_t)m.cnt * sd.n / (min(groups, (int64_t)CL * W) * 32) : sd.n;
     hdr->mode = ok && left <= sd.cap ? 1u : 0u;
   }
 }
 
-constexpr int kSvThreads = 256;
-constexpr int kSvWarps = kSvThreads / 32;
+constexpr int kSvThreads = kSvWarps * 32;
 template <int DT>
 constexpr int sv_items() { return DT == DT_F64 ? 4 : 8; }
 
@@ -448,8 +457,9 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
   using V = RawPt<DT>;
   __shared__ float4 tab[2 * (R + 2)];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const SieveSet sd = j.sieve;
-  const int64_t unit = (int64_t)blockIdx.x * kSvWarps + warp;
+  const int set = j.sv_sets ? j.sv_cta[blockIdx.x] : 0;
+  const SieveSet sd = j.sv_sets ? j.sv_sets[set] : j.sieve;
+  const int64_t unit = (int64_t)(blockIdx.x - sd.cta0) * kSvWarps + warp;   // of the set
   const int64_t a0 = unit * sd.len;
   // before the table is there: the head of every unit into L2 (input only)
   if (a0 < sd.n) {
@@ -463,9 +473,9 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
     }
   }
   griddep_enter();
-  const SieveHdr hdr = w.sv_hdr[0];
+  const SieveHdr hdr = w.sv_hdr[set];
   if (hdr.mode == 0) return;
-  for (int i = tid; i < 2 * (R + 2); i += kSvThreads) tab[i] = w.sv_tab[i];
+  for (int i = tid; i < 2 * (R + 2); i += kSvThreads) tab[i] = w.sv_tab[(size_t)set * 2 * (R + 2) + i];
   __syncthreads();
   if (a0 >= sd.n) return;
   const uint32_t cnt = (uint32_t)min((int64_t)sd.len, sd.n - a0);
@@ -532,7 +542,7 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
     load(buf[0], i0 + 2 * U * 32);
     if (i0 + U * 32 < cnt) test(buf[1], i0 + U * 32);
   }
-  if (lane == 0) w.sv_cnt[unit] = nout;
+  if (lane == 0) w.sv_cnt[(size_t)blockIdx.x * kSvWarps + warp] = nout;
 }
 
 // Listed points of the set gathered in index order; outside the polygon of
@@ -541,7 +551,8 @@ template <int DT, int R, int CL>
 __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
   griddep_enter();
   extern __shared__ __align__(16) unsigned char smem[];
-  TabSmem<R>& m = *reinterpret_cast<TabSmem<R>*>(smem);
+  using M = TabSmem<R, kTabThreads>;
+  M& m = *reinterpret_cast<M*>(smem);
   using P = typename PointT<DT>::T;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = blockIdx.x % CL;
@@ -568,7 +579,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
     __syncthreads();
     uint32_t pre = x - sum;
 #pragma unroll
-    for (int q = 0; q < kTabWarps; q++) { const uint32_t v = m.pre[q]; pre += q < warp ? v : 0u; total += v; }
+    for (int q = 0; q < M::W; q++) { const uint32_t v = m.pre[q]; pre += q < warp ? v : 0u; total += v; }
 #pragma unroll
     for (uint32_t q = 0; q < PU; q++) { m.upre[tid * PU + q] = pre; pre += c[q]; }
     __syncthreads();
@@ -595,7 +606,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
   }
   // items in index order: CTA, warp, k, lane
   const uint32_t cper = ((total + CL - 1) / CL + 31) / 32 * 32;           // per CTA
-  const uint32_t wper = ((cper + kTabWarps - 1) / kTabWarps + 31) / 32 * 32;   // per warp: 32 kTabItems at most
+  const uint32_t wper = ((cper + M::W - 1) / M::W + 31) / 32 * 32;   // per warp: 32 kTabItems at most
   const uint32_t w0 = rank * cper + warp * wper;
   const uint32_t w1 = min(min(total, (uint32_t)(rank + 1) * cper), w0 + wper);
   uint32_t g[kTabItems];
@@ -612,7 +623,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
     X[k] = Y[k] = 0.f;
     if ((have >> k) & 1u) valid |= (uint32_t)sieve_view<DT>(j, sd.off + g[k], X[k], Y[k]) << k;
   }
-  const bool ok = build_table<R, CL>(m, X, Y, valid, rank, tab, hdr);
+  const bool ok = build_table<R, CL, kTabThreads>(m, X, Y, valid, rank, tab, hdr);
   uint32_t keep = have;
   if (ok) {
     const SieveHdr h = fresh_hdr(hdr);
@@ -654,22 +665,31 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
 
 constexpr int kSvCluster = 16;                     // CTAs per cluster (more than 8: opt-in)
 constexpr int64_t kSvPrefetch = int64_t(64) << 20;  // bytes k_sieve prefetches while k_table runs
-constexpr int kSvRows = 512;                       // bands per axis
 
 template <int DT>
 int launch_sieve_t(const Job& j, const Ws& w, cudaStream_t st) {
-  constexpr size_t sm = sizeof(TabSmem<kSvRows>);
+  constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
+  constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>);
   static bool once = [] {
-    cudaFuncSetAttribute(k_table<DT, kSvRows, kSvCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_refine<DT, kSvRows, kSvCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_table<DT, kSvRows, kSvCluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_refine<DT, kSvRows, kSvCluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_table<DT, R, CL, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_table<DT, R, CL, T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if constexpr (DT != DT_F32)
+      cudaFuncSetAttribute(k_table<DT, RB, 1, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
     return true;
   }();
   (void)once;
-  launch_pdl_cluster(k_table<DT, kSvRows, kSvCluster>, kSvCluster, kTabThreads, kSvCluster, sm, st, j, w);
-  launch_pdl(k_sieve<DT, kSvRows>, (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st, j, w);
-  launch_pdl_cluster(k_refine<DT, kSvRows, kSvCluster>, kSvCluster, kTabThreads, kSvCluster, sm, st, j, w);
+  if constexpr (DT != DT_F32) {              // no batches of float32 vectors
+    if (j.sv_sets) {
+      launch_pdl(k_table<DT, RB, 1, TB>, j.nsets, TB, smb, st, j, w);
+      launch_pdl(k_sieve<DT, RB>, j.sv_nctas, kSvThreads, 0, st, j, w);
+      return 2;
+    }
+  }
+  launch_pdl_cluster(k_table<DT, R, CL, T>, CL, T, CL, sm, st, j, w);
+  launch_pdl(k_sieve<DT, R>, (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st, j, w);
+  launch_pdl_cluster(k_refine<DT, R, CL>, CL, T, CL, sm, st, j, w);
   return 3;
 }
 
@@ -688,7 +708,17 @@ SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms) {
   return s;
 }
 
-size_t sieve_table_bytes() { return sizeof(float4) * 2 * (kSvRows + 2); }
+SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0) {
+  SieveSet s{};
+  s.off = off;
+  s.n = n;
+  s.len = kSvBatchLen;
+  const int64_t units = (n + kSvBatchLen - 1) / kSvBatchLen;
+  s.nunit = units <= kSvBatchUnits ? (int32_t)units : 0;
+  s.cap = kSetMax / 4 * 3;
+  s.cta0 = cta0;
+  return s;
+}
 
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st) {
   int nk;

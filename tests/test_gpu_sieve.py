@@ -114,3 +114,32 @@ def test_larger_sets():
     for kind, n in (("square", 5_000_011), ("disk", 5_000_011), ("shell", 3_000_017), ("idisk", 4_000_037)):
         p = KINDS[kind](n, 11)
         assert np.array_equal(run(p), oracle.hull(p)), kind
+
+
+def test_batches():
+    """Sets of every route in one call: whole, sieved, refused (circles), over the sieve's unit limit."""
+    rng = np.random.default_rng(3)
+    sizes = [16_383, 16_384, 18_433, 40_000, 65_537, 131_072, 262_144, 700, 20_000, 0, 33_333]
+    for kinds in (["square", "disk", "gauss"], ["disk", "circle", "shell", "dupes", "sliver"], ["idisk", "isquare", "igrid"],
+                  ["iwide", "idisk"]):
+        sets = [np.ascontiguousarray(KINDS[kinds[int(rng.integers(len(kinds)))]](max(n, 1), i + 1)[:n])
+                for i, n in enumerate(sizes * 3)]
+        off = np.concatenate([[0], np.cumsum([len(p) for p in sets])])
+        for _ in range(2):
+            got = cch.hull_batched(torch.from_numpy(np.concatenate(sets)).to(DEV), off)
+            for i, (p, h) in enumerate(zip(sets, got)):
+                assert np.array_equal(h.cpu().numpy(), oracle.hull(p)), (kinds, i, len(p))
+
+
+def test_batch_bad_and_large():
+    big, bad = inputs.disk_f64(2_200_000, 4), inputs.disk_f64(90_001, 5)
+    bad[777] = [0.01, np.nan]
+    sets = [inputs.disk_f64(50_000, 1), bad, big, inputs.circle_f64(30_000, 2), inputs.square_f64(400_001, 3)]
+    off = np.concatenate([[0], np.cumsum([len(p) for p in sets])])
+    idx = torch.zeros(int(off[-1]), dtype=torch.int32, device=DEV)
+    cnt = torch.zeros(len(sets), dtype=torch.int32, device=DEV)
+    cch.hull_batched_async(torch.from_numpy(np.concatenate(sets)).to(DEV), off, idx, cnt)
+    c = cnt.cpu().numpy()
+    assert c[1] == -3
+    for i in (0, 2, 3, 4):
+        assert np.array_equal(idx[int(off[i]):int(off[i]) + int(c[i])].cpu().numpy(), oracle.hull(sets[i])), i
