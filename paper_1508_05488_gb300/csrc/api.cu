@@ -404,6 +404,7 @@ int cch_hull(const void* points, int64_t n, int dtype, int32_t* out_idx, int32_t
   if (n <= kSetOne) return run_set(set_job(points, nullptr, n, dtype, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(points, n, dtype, out_idx, out_count, 0);
   j.sieve = sieve_set(0, n, dtype, sm_count());
+  j.fast_sort = 1;
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
 
@@ -519,6 +520,7 @@ int cch_hull_f32soa(const float* x, const float* y, int64_t n, int32_t* out_idx,
   Job j = single_job(x, n, DT_F32, out_idx, out_count, 0);
   j.ys = y;
   j.sieve = sieve_set(0, n, DT_F32, sm_count());
+  j.fast_sort = 1;
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
 

@@ -133,6 +133,9 @@ enum : int {
   CT_SORT_TILE0,                       // + pass
   CT_SPA_TILE = CT_SORT_TILE0 + kSortPasses,
   CT_OUT_TILE, CT_OUT_DONE,
+  CT_FAST_TILE0,                       // + pass of k_big's sort by quantised keys
+  CT_FAST_RUNS = CT_FAST_TILE0 + 4,    // its runs out of order, and whether one is too long: found by the
+  CT_FAST_FAIL, CT_FAST_FAIL2,         //   check, found by the repair (apart: some CTAs read the first late)
   CT_SORT_TOTAL,                       // plan results
   CT_SPA_TOTAL,
   CT_CHAIN_TOTAL,
@@ -213,6 +216,7 @@ struct Job {
   int64_t chunk1_len;   // a1 chunk length (points), multiple of 256
   uint32_t epoch;       // look-back flag epoch of this call (1..0xFFFF)
   uint32_t opts;        // OPT_* bits
+  uint32_t fast_sort;   // a single set whose multi-block sort may go by quantised keys
   Tune tune;            // run-time choices (the same results with any valid choice)
   const SetDesc* sets;  // device array, or nullptr -> use `one`
   SetDesc one;
