@@ -53,8 +53,9 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kTabThreads = 1024;                   // of k_refine, and of k_table on a single set
-constexpr int kTabBatchThreads = 512;               // of k_table on a batch's sets
-constexpr int kTabItems = 8;                        // sample points per thread at most
+constexpr int kTabBatchThreads = 256;               // of k_table on a batch's sets: 4096 sample points each, four
+                                                    // sets per SM (512 threads, two: 37 us for 409 sets, 30 so)
+constexpr int kTabItems = 8, kTabBatchItems = 16;   // points per thread at most
 constexpr int kPeel = 40;                           // peeling rounds at most
 constexpr uint32_t kPlain = 2048;                   // lists up to this size go to k_set as they are
 
@@ -153,19 +154,19 @@ __device__ __forceinline__ uint32_t warp_incl_sum(uint32_t x) {
   return x;
 }
 
-// Polygon tables of the cluster's points (kTabItems views per thread at most, `valid`
+// Polygon tables of the cluster's points (NI views per thread, `valid`
 // bit k: item k), by every thread of the cluster.  They go to `tab` and `hdr`
 // (global memory) and are visible to the cluster on return; false where there
 // are none.
-template <int R, int CL, int T>
-__device__ bool build_table(TabSmem<R, T>& m, const float (&X)[kTabItems], const float (&Y)[kTabItems], uint32_t valid,
+template <int R, int CL, int T, int NI>
+__device__ bool build_table(TabSmem<R, T>& m, const float (&X)[NI], const float (&Y)[NI], uint32_t valid,
                             int rank, float4* tab, SieveHdr* hdr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // extremes: per side the smallest v (and the smallest u among them)
   {
     uint64_t e[4] = {~0ull, ~0ull, ~0ull, ~0ull};
 #pragma unroll
-    for (int k = 0; k < kTabItems; k++) {
+    for (int k = 0; k < NI; k++) {
       if ((valid >> k) & 1u) {
         const uint32_t ox = f32_order(X[k]), oy = f32_order(Y[k]);
         e[0] = min(e[0], kw(ox, oy));
@@ -215,7 +216,7 @@ __device__ bool build_table(TabSmem<R, T>& m, const float (&X)[kTabItems], const
   }
   // the smallest v of every band, then its u (any point that holds the minimum)
 #pragma unroll
-  for (int k = 0; k < kTabItems; k++) {
+  for (int k = 0; k < NI; k++) {
     if ((valid >> k) & 1u) {
       const int b = min((int)((Y[k] - y0) * by), R - 1), c = min((int)((X[k] - x0) * bx), R - 1);
       const uint32_t ox = f32_order(X[k]), oy = f32_order(Y[k]);
@@ -228,7 +229,7 @@ __device__ bool build_table(TabSmem<R, T>& m, const float (&X)[kTabItems], const
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < kTabItems; k++) {
+  for (int k = 0; k < NI; k++) {
     if ((valid >> k) & 1u) {
       const int b = min((int)((Y[k] - y0) * by), R - 1), c = min((int)((X[k] - x0) * bx), R - 1);
       const uint32_t ox = f32_order(X[k]), oy = f32_order(Y[k]);
@@ -401,7 +402,7 @@ __device__ __forceinline__ SieveHdr fresh_hdr(const SieveHdr* h) {
 }
 
 // Table of each set from a sample spread over it in runs of 32 points.
-template <int DT, int R, int CL, int T>
+template <int DT, int R, int CL, int T, int NI>
 __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   griddep_enter();
   extern __shared__ __align__(16) unsigned char smem[];
@@ -418,19 +419,19 @@ __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
     return;
   }
   // at most n / 8 points in runs of 32
-  const int64_t groups = min((int64_t)CL * W * kTabItems, max(sd.n / 256, (int64_t)1));
+  const int64_t groups = min((int64_t)CL * W * NI, max(sd.n / 256, (int64_t)1));
   const int64_t step = sd.n / groups;
-  float X[kTabItems], Y[kTabItems];
+  float X[NI], Y[NI];
   uint32_t valid = 0;
 #pragma unroll
-  for (int k = 0; k < kTabItems; k++) {
+  for (int k = 0; k < NI; k++) {
     const int64_t g = ((int64_t)k * CL + rank) * W + warp;
     X[k] = Y[k] = 0.f;
     if (g < groups) valid |= (uint32_t)sieve_view<DT>(j, sd.off + g * step + lane, X[k], Y[k]) << k;
   }
   // the sample is here: k_sieve's CTAs may start and prefetch
   griddep_release();
-  const bool ok = build_table<R, CL, T>(m, X, Y, valid, rank, tab, hdr);
+  const bool ok = build_table<R, CL, T, NI>(m, X, Y, valid, rank, tab, hdr);
   // what is left of the first item of every thread tells whether the sieve pays
   uint32_t outn = 0;
   if (ok) {
@@ -623,7 +624,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
     X[k] = Y[k] = 0.f;
     if ((have >> k) & 1u) valid |= (uint32_t)sieve_view<DT>(j, sd.off + g[k], X[k], Y[k]) << k;
   }
-  const bool ok = build_table<R, CL, kTabThreads>(m, X, Y, valid, rank, tab, hdr);
+  const bool ok = build_table<R, CL, kTabThreads, kTabItems>(m, X, Y, valid, rank, tab, hdr);
   uint32_t keep = have;
   if (ok) {
     const SieveHdr h = fresh_hdr(hdr);
@@ -671,23 +672,23 @@ int launch_sieve_t(const Job& j, const Ws& w, cudaStream_t st) {
   constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
   constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>);
   static bool once = [] {
-    cudaFuncSetAttribute(k_table<DT, R, CL, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_table<DT, R, CL, T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if constexpr (DT != DT_F32)
-      cudaFuncSetAttribute(k_table<DT, RB, 1, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
+      cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
     return true;
   }();
   (void)once;
   if constexpr (DT != DT_F32) {              // no batches of float32 vectors
     if (j.sv_sets) {
-      launch_pdl(k_table<DT, RB, 1, TB>, j.nsets, TB, smb, st, j, w);
+      launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
       launch_pdl(k_sieve<DT, RB>, j.sv_nctas, kSvThreads, 0, st, j, w);
       return 2;
     }
   }
-  launch_pdl_cluster(k_table<DT, R, CL, T>, CL, T, CL, sm, st, j, w);
+  launch_pdl_cluster(k_table<DT, R, CL, T, kTabItems>, CL, T, CL, sm, st, j, w);
   launch_pdl(k_sieve<DT, R>, (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st, j, w);
   launch_pdl_cluster(k_refine<DT, R, CL>, CL, T, CL, sm, st, j, w);
   return 3;
