@@ -182,7 +182,10 @@ int cch_hull_stages(const void *points, int64_t n, int dtype, uint32_t opts,
  * records only around the stages whose bit is set in mask (bit k: stage k;
  * the others read as 0), which keeps the events' own cost out of the rest
  * of the pipeline; mask 0 stops recording.  Small sets are computed by one
- * kernel each, outside these stages.
+ * kernel each, outside these stages.  Larger sets that take the one-pass
+ * sieve spend theirs in the stages its kernels stand for: the sample's table
+ * in (1), the pass over the points in (2), the gathering of its list in (3),
+ * the hull of the list in (6).
  */
 int cch_profile(int enable);
 int cch_profile_stages(uint32_t mask);

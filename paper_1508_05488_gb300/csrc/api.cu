@@ -84,7 +84,7 @@ Layout layout(const Dims& d, char* base) {
   L.w.out_start = (uint32_t*)take(4 * (4 * (size_t)d.nsets + 1));
   L.w.stairs = (uint32_t*)take(4 * 4 * (size_t)kStairB * d.nsets);
   L.w.sv_hdr = (SieveHdr*)take(sizeof(SieveHdr) * d.nsets);
-  L.w.sv_tab = (float4*)take(2 * sizeof(float4) * std::max<size_t>(kSvRows + 2, (size_t)(kSvBatchRows + 2) * d.nsets));
+  L.w.sv_tab = (float4*)take(2 * sizeof(float4) * std::max<size_t>(kSvRefineRows + 2, (size_t)(kSvBatchRows + 2) * d.nsets));
   L.w.sv_cnt = (uint32_t*)take(4 * std::max<size_t>(kSvMaxUnits, kSvWarps * ((size_t)d.N / (kSvWarps * kSvBatchLen) + d.nsets + 1)));
   L.total = o;
   return L;
@@ -99,6 +99,8 @@ struct Workspace {
   char* dev_tab = nullptr;           // their device copy
   size_t tab_bytes = 0;              // size of both
   cudaEvent_t tab_done = nullptr;    // staging buffer free again
+  cudaStream_t side = nullptr;       // the pipeline beside k_set (run)
+  cudaEvent_t fork = nullptr, join = nullptr;
   void* h2d = nullptr;               // device copy of host points (cch_hull_host)
   size_t h2d_bytes = 0;
   int32_t* dcount = nullptr;         // device counts (cch_hull_host)
@@ -113,15 +115,22 @@ std::atomic<uint64_t> g_launches{0};
 // Optional stage timing: CUDA events around the stages of every call, read
 // back (and summed) by cch_profile_read.
 constexpr int kStages = 8;   // a1, stairs, a2, gather, small path, multi-block path, chain, blocked SPA
-struct ProfRec { cudaEvent_t ev[kStages + 1]; uint32_t mask; };
+// The sieve's kernels, timed with the stages they stand for: k_table (sample),
+// k_sieve (a2), k_refine (gather) and k_set on the lists (chain hull, output).
+constexpr int kSieveStages = 4, kSieveStage[kSieveStages] = {1, 2, 3, 6};
+struct ProfRec { cudaEvent_t ev[kStages + 1], sv[kSieveStages + 1]; uint32_t mask; bool sieve; };
 uint32_t g_prof = 0;   // stages whose boundaries get events (bit k: stage k)
 std::vector<ProfRec> g_prof_pending, g_prof_free;
 
 cudaEvent_t* prof_begin(ProfRec& rec) {
   if (!g_prof) return nullptr;
   if (!g_prof_free.empty()) { rec = g_prof_free.back(); g_prof_free.pop_back(); }
-  else for (auto& e : rec.ev) cudaEventCreate(&e);
+  else {
+    for (auto& e : rec.ev) cudaEventCreate(&e);
+    for (auto& e : rec.sv) cudaEventCreate(&e);
+  }
   rec.mask = g_prof;
+  rec.sieve = false;
   return rec.ev;
 }
 int g_sms = 0;
@@ -162,6 +171,14 @@ int acquire(cudaStream_t stream, const Dims& d, Workspace* ws) {
       return CCH_ERR_NOMEM;
     }
     if (cudaMemsetAsync(ws->dev, 0, L.total, stream) != cudaSuccess) return CCH_ERR_CUDA;
+    if (!ws->side) {                 // optional: without it everything stays on the caller's stream
+      if (cudaStreamCreateWithFlags(&ws->side, cudaStreamNonBlocking) != cudaSuccess ||
+          cudaEventCreateWithFlags(&ws->fork, cudaEventDisableTiming) != cudaSuccess ||
+          cudaEventCreateWithFlags(&ws->join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        ws->join = nullptr;
+      }
+    }
     ws->bytes = L.total;
     ws->cap = c;
     ws->epoch = 0;
@@ -281,14 +298,38 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   j.epoch = ws->epoch;
   if (cudaMemsetAsync(ws->dev, 0, L.ctl_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
   if (stages) { j.r1_idx = stages->r1_idx; j.r1_region = stages->r1_region; }
-  Launch La{stream, grid_cap(), j.tune.cls_per_sm * sm_count()};
   ProfRec rec{};
   cudaEvent_t* ev = prof_begin(rec);
+  // The sieve's lists, then k_set on them and the pipeline, which has nothing
+  // to do for a sieved call: each of its nine launches still waits for the one
+  // before it, 10 us in all after k_set, so it runs on a stream of the
+  // workspace beside k_set and joins the caller's (not when stages are timed).
+  bool side = false;
+  if (j.sieve.nunit || j.sv_sets) {
+    rec.sieve = true;
+    // sieve event k marks the start of its stage k (and the end of k - 1)
+    auto mark_sv = [&](int k) {
+      if (ev && ((k < kSieveStages && (rec.mask >> kSieveStage[k]) & 1u) || (k > 0 && (rec.mask >> kSieveStage[k - 1]) & 1u)))
+        cudaEventRecord(rec.sv[k], stream);
+    };
+    mark_sv(0);
+    nk += launch_table(j, L.w, stream);
+    mark_sv(1);
+    nk += launch_sieve(j, L.w, stream);
+    mark_sv(2);
+    nk += launch_refine(j, L.w, stream);
+    side = !ev && !j.sv_sets && ws->join;
+    if (side && (cudaEventRecord(ws->fork, stream) != cudaSuccess ||
+                 cudaStreamWaitEvent(ws->side, ws->fork, 0) != cudaSuccess)) return CCH_ERR_CUDA;
+    mark_sv(3);
+    nk += launch_set_list(j, L.w, stream);
+    mark_sv(4);
+  }
+  Launch La{side ? ws->side : stream, grid_cap(), j.tune.cls_per_sm * sm_count()};
   // event k marks the start of stage k (and the end of stage k - 1)
   auto mark = [&](int k) {
     if (ev && ((rec.mask >> k) & 1u || (k > 0 && (rec.mask >> (k - 1)) & 1u))) cudaEventRecord(ev[k], stream);
   };
-  if (j.sieve.nunit || j.sv_sets) nk += launch_sieve(j, L.w, stream);
   mark(0);
   nk += launch_extremes(j, L.w, La);
   mark(1);
@@ -304,6 +345,8 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   mark(6);
   nk += launch_chain(j, L.w, La);
   mark(7);
+  if (side && (cudaEventRecord(ws->join, ws->side) != cudaSuccess ||
+               cudaStreamWaitEvent(stream, ws->join, 0) != cudaSuccess)) return CCH_ERR_CUDA;
   if (stages) {
     if (j.opts & OPT_BLOCKED_SPA) nk += launch_spa_blocked(j, L.w, stages->spa_idx, stream);
     else { launch_extract_spa(j, L.w, stages->spa_idx, stream); nk++; }
@@ -582,6 +625,13 @@ int cch_profile_read(double* stage_ms, int max_stages, int64_t* calls) {
       cudaEventElapsedTime(&ms, rec.ev[k], rec.ev[k + 1]);
       stage_ms[k] += ms;
     }
+    for (int q = 0; rec.sieve && q < kSieveStages; q++) {
+      const int k = kSieveStage[q];
+      if (!((rec.mask >> k) & 1u) || k >= max_stages) continue;
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, rec.sv[q], rec.sv[q + 1]);
+      stage_ms[k] += ms;
+    }
     g_prof_free.push_back(rec);
     n++;
   }
@@ -642,6 +692,9 @@ void cch_release_workspace(void) {
     if (ws->host_tab) cudaFreeHost(ws->host_tab);
     if (ws->dev_tab) cudaFree(ws->dev_tab);
     if (ws->tab_done) cudaEventDestroy(ws->tab_done);
+    if (ws->side) cudaStreamDestroy(ws->side);
+    if (ws->fork) cudaEventDestroy(ws->fork);
+    if (ws->join) cudaEventDestroy(ws->join);
     if (ws->h2d) cudaFree(ws->h2d);
     if (ws->dcount) cudaFree(ws->dcount);
     if (ws->didx) cudaFree(ws->didx);

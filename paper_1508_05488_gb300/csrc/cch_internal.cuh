@@ -193,7 +193,7 @@ constexpr int kSvWarps = 8;            // warps, hence units, per k_sieve CTA
 // A batch's larger sets: units of kSvBatchLen points, kSvBatchUnits per set at
 // most (larger sets take the pipeline), tables of kSvBatchRows bands.
 constexpr int kSvBatchLen = 2048, kSvBatchUnits = 1024, kSvBatchRows = 256;
-constexpr int kSvRows = 512;           // bands per axis of a single set's table
+constexpr int kSvRows = 256, kSvRefineRows = 512;   // bands per axis of a single set's tables
 // Device side of it: the maps of the bands (of Y: s[0] Y + o[0], of X: s[1] X +
 // o[1]), whether the sieve runs (mode) and the number of listed points.
 struct alignas(16) SieveHdr {
@@ -985,14 +985,13 @@ __device__ __forceinline__ void griddep_enter() { asm volatile("griddepcontrol.w
 __device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Whether the sieve takes the set (k_sieve.cu).  The flag is written by
-// k_refine, which k_set waits for before it releases the pipeline.
+// k_refine (a batch: k_set), which the pipeline's first kernel comes after.
 __device__ __forceinline__ bool sieved(const Ws& w) { return *(volatile const uint32_t*)(w.ctr + CT_SIEVED) != 0; }
 // The same at the start of a kernel of the pipeline, before its griddep_enter:
 // each starts when every CTA of the kernel before it has left or released it,
 // so the flag is there.  Where it is set the kernel has nothing to do: it lets
 // its successor start at once, and one CTA waits, so that the kernel still
-// completes after the one before it.  These nine launches run beside k_set and
-// add 5 us to a call where each waiting for the last one's end added 14.
+// completes after the one before it.
 __device__ __forceinline__ bool sieved_leave(const Ws& w) {
   if (!sieved(w)) return false;
   griddep_release();
@@ -1039,7 +1038,9 @@ int launch_set(const Job& j, int cls, const SetItem* items, int count, bool besi
 int launch_set_list(const Job& j, const Ws& w, cudaStream_t st);   // the sieve's listed points
 SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);
 SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0);
+int launch_table(const Job& j, const Ws& w, cudaStream_t st);
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st);
+int launch_refine(const Job& j, const Ws& w, cudaStream_t st);   // a single set's; a batch has none
 int launch_extremes(const Job& j, const Ws& w, const Launch& L);
 int launch_stairs(const Job& j, const Ws& w, const Launch& L);
 int launch_classify(const Job& j, const Ws& w, const Launch& L);

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   if (MODE != SET_WHOLE || !beside) griddep_enter();
   if constexpr (LIST) {
     if (!sieved(w)) return;
-    griddep_release();                       // the pipeline has nothing to do (sieved_leave)
+    griddep_release();                       // where it follows on this stream, the pipeline only leaves
   }
   if constexpr (MODE == SET_WHOLE) griddep_release();
   constexpr int CAP = SetClass<C>::CAP, T = SetClass<C>::T, NB = SetClass<C>::NB, NW = T / 32;

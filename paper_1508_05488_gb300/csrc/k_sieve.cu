@@ -668,30 +668,50 @@ constexpr int kSvCluster = 16;                     // CTAs per cluster (more tha
 constexpr int64_t kSvPrefetch = int64_t(64) << 20;  // bytes k_sieve prefetches while k_table runs
 
 template <int DT>
-int launch_sieve_t(const Job& j, const Ws& w, cudaStream_t st) {
+int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
   constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
   constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>);
+  if (j.sv_sets) {
+    if constexpr (DT != DT_F32) {            // no batches of float32 vectors
+      static bool once = [] {
+        cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
+        return true;
+      }();
+      (void)once;
+      launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
+    }
+    return 1;
+  }
   static bool once = [] {
     cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if constexpr (DT != DT_F32)
-      cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
     return true;
   }();
   (void)once;
-  if constexpr (DT != DT_F32) {              // no batches of float32 vectors
-    if (j.sv_sets) {
-      launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
-      launch_pdl(k_sieve<DT, RB>, j.sv_nctas, kSvThreads, 0, st, j, w);
-      return 2;
-    }
-  }
   launch_pdl_cluster(k_table<DT, R, CL, T, kTabItems>, CL, T, CL, sm, st, j, w);
-  launch_pdl(k_sieve<DT, R>, (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st, j, w);
-  launch_pdl_cluster(k_refine<DT, R, CL>, CL, T, CL, sm, st, j, w);
-  return 3;
+  return 1;
+}
+
+template <int DT>
+int launch_sieve_t(const Job& j, const Ws& w, cudaStream_t st) {
+  static_assert(kSvRows == kSvBatchRows, "one k_sieve for both");
+  launch_pdl(k_sieve<DT, kSvRows>, j.sv_sets ? j.sv_nctas : (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st,
+             j, w);
+  return 1;
+}
+
+template <int DT>
+int launch_refine_t(const Job& j, const Ws& w, cudaStream_t st) {
+  constexpr int CL = kSvCluster, R = kSvRefineRows;
+  constexpr size_t sm = sizeof(TabSmem<R, kTabThreads>);
+  static bool once = [] {
+    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return true;
+  }();
+  (void)once;
+  launch_pdl_cluster(k_refine<DT, R, CL>, CL, kTabThreads, CL, sm, st, j, w);
+  return 1;
 }
 
 }  // namespace
@@ -721,12 +741,20 @@ SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0) {
   return s;
 }
 
+int launch_table(const Job& j, const Ws& w, cudaStream_t st) {
+  return j.dtype == DT_F64 ? launch_table_t<DT_F64>(j, w, st)
+         : j.dtype == DT_F32 ? launch_table_t<DT_F32>(j, w, st) : launch_table_t<DT_I32>(j, w, st);
+}
+
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st) {
-  int nk;
-  if (j.dtype == DT_F64) nk = launch_sieve_t<DT_F64>(j, w, st);
-  else if (j.dtype == DT_F32) nk = launch_sieve_t<DT_F32>(j, w, st);
-  else nk = launch_sieve_t<DT_I32>(j, w, st);
-  return nk + launch_set_list(j, w, st);
+  return j.dtype == DT_F64 ? launch_sieve_t<DT_F64>(j, w, st)
+         : j.dtype == DT_F32 ? launch_sieve_t<DT_F32>(j, w, st) : launch_sieve_t<DT_I32>(j, w, st);
+}
+
+int launch_refine(const Job& j, const Ws& w, cudaStream_t st) {
+  if (j.sv_sets) return 0;
+  return j.dtype == DT_F64 ? launch_refine_t<DT_F64>(j, w, st)
+         : j.dtype == DT_F32 ? launch_refine_t<DT_F32>(j, w, st) : launch_refine_t<DT_I32>(j, w, st);
 }
 
 }  // namespace cch

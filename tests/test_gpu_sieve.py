@@ -143,3 +143,43 @@ def test_batch_bad_and_large():
     assert c[1] == -3
     for i in (0, 2, 3, 4):
         assert np.array_equal(idx[int(off[i]):int(off[i]) + int(c[i])].cpu().numpy(), oracle.hull(sets[i])), i
+
+
+def test_graph_capture():
+    """A captured call (with its fork to the workspace's stream) replayed on other points."""
+    n = 300_007
+    s = torch.cuda.Stream()
+    pts = torch.zeros((n, 2), dtype=torch.float64, device=DEV)
+    idx = torch.zeros(n, dtype=torch.int32, device=DEV)
+    cnt = torch.zeros(1, dtype=torch.int32, device=DEV)
+    pts.copy_(torch.from_numpy(inputs.disk_f64(n, 1)))
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        cch.hull_async(pts, idx, cnt)                    # the workspace
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        cch.hull_async(pts, idx, cnt)
+    for kind, seed in (("square", 2), ("disk", 3), ("gauss", 4), ("shell", 5)):
+        p = KINDS[kind](n, seed)
+        pts.copy_(torch.from_numpy(np.ascontiguousarray(p)))
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(idx[:int(cnt.item())].cpu().numpy(), oracle.hull(p)), kind
+
+
+def test_streams_at_once():
+    """Sieved and refused sets on several streams, each with its own workspace and side stream."""
+    sets = [KINDS[k](150_001 + 7 * i, i + 1) for i, k in enumerate(["disk", "circle", "square", "shell", "gauss", "circle"])]
+    pts = [torch.from_numpy(np.ascontiguousarray(p)).to(DEV) for p in sets]
+    streams = [torch.cuda.Stream() for _ in sets]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        outs = []
+        for p, s in zip(pts, streams):
+            with torch.cuda.stream(s):
+                outs.append(cch.hull_async(p))
+        torch.cuda.synchronize()
+        for p, (idx, cnt) in zip(sets, outs):
+            assert np.array_equal(idx[:int(cnt.item())].cpu().numpy(), oracle.hull(p))
