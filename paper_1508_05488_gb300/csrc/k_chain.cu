@@ -59,6 +59,15 @@ struct GlobAcc {
   }
 };
 
+// Threads of k_chain_local.  A block's 160 KB of shared memory leave one CTA on
+// an SM, so its warps are all there is to hide the orientation tests' latency.
+// 256 / 512 / 1024 threads: 108 / 96 / 90 us on a circle of 2M points, and the
+// whole call on the degenerate 20M set, whose blocks peel for many rounds,
+// 1431 / 1405 / 1500 us.
+constexpr int kChThreads = 512;
+constexpr int kChWarps = kChThreads / 32;
+constexpr int kChPer = kChainBlk / kChThreads;
+
 // Asynchronous global -> shared copy of B (8 or 16) bytes, both B-aligned.
 template <int B>
 __device__ __forceinline__ void cp_async_copy(void* dst, const void* src) {
@@ -69,7 +78,7 @@ __device__ __forceinline__ void cp_async_copy(void* dst, const void* src) {
 }
 
 
-// Exclusive prefix sum of one value per thread over the CTA; sh[kWarps]
+// Exclusive prefix sum of one value per thread over the CTA; sh[kChWarps]
 // receives the total.  Ends with the CTA synchronised.
 __device__ __forceinline__ int block_excl_sum(int v, int* sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -83,26 +92,26 @@ __device__ __forceinline__ int block_excl_sum(int v, int* sh) {
   if (lane == 31) sh[warp] = x;
   __syncthreads();
   int pre = x - v, tot = 0;
-  for (int q = 0; q < kWarps; q++) {
+  for (int q = 0; q < kChWarps; q++) {
     if (q < warp) pre += sh[q];
     tot += sh[q];
   }
   __syncthreads();
-  if (threadIdx.x == 0) sh[kWarps] = tot;
+  if (threadIdx.x == 0) sh[kChWarps] = tot;
   __syncthreads();
   return pre;
 }
 
 // Positions i < m with al[i] != 0, in order, into out; returns their count.
 __device__ __forceinline__ int block_compact(const uint8_t* al, int m, uint16_t* out, int* sh) {
-  const int per = (m + kThreads - 1) / kThreads;
+  const int per = (m + kChThreads - 1) / kChThreads;
   const int i0 = threadIdx.x * per;
   int c = 0;
   for (int q = 0; q < per; q++) c += (i0 + q < m && al[i0 + q]) ? 1 : 0;
   int pre = block_excl_sum(c, sh);
   for (int q = 0; q < per; q++)
     if (i0 + q < m && al[i0 + q]) out[pre++] = (uint16_t)(i0 + q);
-  const int n = sh[kWarps];
+  const int n = sh[kChWarps];
   __syncthreads();
   return n;
 }
@@ -119,7 +128,7 @@ __device__ void chain_set_output(const Job& j, const Ws& w, const SetDesc& sd, i
   for (int r = 0; r < 4; r++) {
     const uint32_t nr = __ldcg(&c.nal[r]);
     const uint32_t* src = w.cprev + chain_base(sd, s, c, r);
-    for (uint32_t k = threadIdx.x; k < nr; k += kThreads) j.out_idx[sd.off + off + k] = (int32_t)__ldcg(src + k);
+    for (uint32_t k = threadIdx.x; k < nr; k += kChThreads) j.out_idx[sd.off + off + k] = (int32_t)__ldcg(src + k);
     off += nr;
   }
   if (threadIdx.x == 0) j.out_counts[sd.id] = (int32_t)off;
@@ -128,11 +137,11 @@ __device__ void chain_set_output(const Job& j, const Ws& w, const SetDesc& sd, i
 template <int DT>
 constexpr size_t chain_local_smem() {
   return (size_t)kChainBlk * (sizeof(typename PT<DT>::T) + (DT == DT_F64 ? 16 : 0) + 2 + 2 + 2 + 1) +
-         2 * kThreads * sizeof(int);
+         2 * kChThreads * sizeof(int);
 }
 
 template <int DT>
-__global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
+__global__ void __launch_bounds__(kChThreads) k_chain_local(Job j, Ws w) {
   if (sieved_leave(w)) return;
   griddep_enter();
   using P = typename PT<DT>::T;
@@ -143,10 +152,10 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
   uint16_t* nx = pv + kChainBlk;
   uint16_t* stk = nx + kChainBlk;
   int* gh = reinterpret_cast<int*>(stk + kChainBlk);
-  int* gt = gh + kThreads;
-  uint8_t* al = reinterpret_cast<uint8_t*>(gt + kThreads);
+  int* gt = gh + kChThreads;
+  uint8_t* al = reinterpret_cast<uint8_t*>(gt + kChThreads);
   __shared__ P pred;
-  __shared__ int sh_cnt[kWarps + 1];
+  __shared__ int sh_cnt[kChWarps + 1];
   __shared__ int sh_last;
 
   const uint32_t total = w.ctr[CT_CHAIN_TOTAL];
@@ -164,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
     const int m = (int)min((uint32_t)kChainBlk, L - p0);
     // the block's points straight into shared memory (all copies in
     // flight at once); the chain's two extremes come from the set's record
-    for (int i = threadIdx.x; i < m; i += kThreads) {
+    for (int i = threadIdx.x; i < m; i += kChThreads) {
       const uint32_t p = p0 + i;
       if (p != 0 && p != L - 1) cp_async_copy<sizeof(P)>(&sp[i], &cp[cb + p]);
     }
@@ -183,14 +192,14 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
     }
     if constexpr (DT == DT_F64) {
       __syncthreads();
-      for (int i = threadIdx.x; i < m; i += kThreads) sf[i] = f64_split4(sp[i]);
+      for (int i = threadIdx.x; i < m; i += kChThreads) sf[i] = f64_split4(sp[i]);
     }
     if (threadIdx.x == 0 && p0 > 0) pred = cp[cb + p0 - 1];
     __syncthreads();
 
     SmemAcc<DT> acc{sp, sf, pv, nx, al, flag};
     // identical neighbours: the first index stays
-    for (int i = threadIdx.x; i < m; i += kThreads) {
+    for (int i = threadIdx.x; i < m; i += kChThreads) {
       bool dup;
       if (i > 0) dup = same_pt<DT>(sp[i], sp[i - 1]);
       else dup = p0 > 0 && same_pt<DT>(sp[0], pred);
@@ -209,7 +218,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
     int n = block_compact(al, m, cur, sh_cnt);
     bool conv = false;
     for (int round = 0; round < kPeelRounds && !conv; round++) {
-      const int per = (n + kThreads - 1) / kThreads;
+      const int per = (n + kChThreads - 1) / kChThreads;
       const int t0 = threadIdx.x * per;
       uint32_t keep = 0;
       for (int q = 0; q < per; q++) {
@@ -221,7 +230,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
       }
       const int nk = __popc(keep);
       int pre = block_excl_sum(nk, sh_cnt);
-      const int n2 = sh_cnt[kWarps];
+      const int n2 = sh_cnt[kChWarps];
       for (int q = 0; q < per; q++) {
         const int t = t0 + q;
         if (t >= n) break;
@@ -236,11 +245,11 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
     if (conv) {
       // links of the convex sequence (held in stk, so that nx is free)
       if (cur != stk) {
-        for (int t = threadIdx.x; t < n; t += kThreads) stk[t] = cur[t];
+        for (int t = threadIdx.x; t < n; t += kChThreads) stk[t] = cur[t];
         __syncthreads();
         cur = stk;
       }
-      for (int t = threadIdx.x; t < n; t += kThreads) {
+      for (int t = threadIdx.x; t < n; t += kChThreads) {
         const int i = cur[t];
         if (t > 0) pv[i] = cur[t - 1];
         if (t + 1 < n) nx[i] = cur[t + 1];
@@ -253,8 +262,8 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
       // not converged: per thread a strict left-turn stack over its 16
       // positions (peeled points skipped), then pairwise merges
       __syncthreads();
-      const int i0 = threadIdx.x * kChainItems;
-      const int i1 = min(m, i0 + kChainItems);
+      const int i0 = threadIdx.x * kChPer;
+      const int i1 = min(m, i0 + kChPer);
       int top = 0;
       for (int i = i0; i < i1; i++) {
         if (!al[i]) continue;
@@ -270,10 +279,10 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
       }
       gh[threadIdx.x] = top ? stk[i0] : -1;
       gt[threadIdx.x] = top ? stk[i0 + top - 1] : -1;
-      for (int step = 1; step < kThreads; step <<= 1) {
+      for (int step = 1; step < kChThreads; step <<= 1) {
         __syncthreads();
         const int t = threadIdx.x;
-        if ((t & (2 * step - 1)) == 0 && t + step < kThreads && (t + step) * kChainItems < m) {
+        if ((t & (2 * step - 1)) == 0 && t + step < kChThreads && (t + step) * kChPer < m) {
           int hl = gh[t], tl = gt[t];
           merge_chains(acc, hl, tl, gh[t + step], gt[t + step]);
           gh[t] = hl;
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
       // the indices of the kept positions but the last, in order, at the
       // start of the chain's link slots (no merge or output pass follows)
       const int nout = block_compact(al, m - 1, stk, sh_cnt);
-      for (int k = threadIdx.x; k < nout; k += kThreads) w.cprev[cb + k] = w.cidx[cb + stk[k]];
+      for (int k = threadIdx.x; k < nout; k += kChThreads) w.cprev[cb + k] = w.cidx[cb + stk[k]];
       __syncthreads();
       if (threadIdx.x == 0) {
         w.ctl[s].nal[r] = (uint32_t)nout;
@@ -301,7 +310,7 @@ __global__ void __launch_bounds__(kThreads) k_chain_local(Job j, Ws w) {
       __syncthreads();
       continue;
     }
-    for (int i = threadIdx.x; i < m; i += kThreads) {
+    for (int i = threadIdx.x; i < m; i += kChThreads) {
       w.calive[cb + p0 + i] = al[i];
       if (al[i]) {
         w.cprev[cb + p0 + i] = p0 + pv[i];
@@ -487,7 +496,7 @@ int launch_chain(const Job& j, const Ws& w, const Launch& L) {
       return true;
     }();
     (void)once;
-    launch_pdl(k_chain_local<DT_F64>, grid, kThreads, sm, L.stream, j, w);
+    launch_pdl(k_chain_local<DT_F64>, grid, kChThreads, sm, L.stream, j, w);
     launch_pdl(k_chain_merge<DT_F64>, gridm, kThreads, 0, L.stream, j, w);
   } else {
     constexpr size_t sm = chain_local_smem<DT_I32>();
@@ -496,7 +505,7 @@ int launch_chain(const Job& j, const Ws& w, const Launch& L) {
       return true;
     }();
     (void)once;
-    launch_pdl(k_chain_local<DT_I32>, grid, kThreads, sm, L.stream, j, w);
+    launch_pdl(k_chain_local<DT_I32>, grid, kChThreads, sm, L.stream, j, w);
     launch_pdl(k_chain_merge<DT_I32>, gridm, kThreads, 0, L.stream, j, w);
   }
   launch_pdl(k_output, grid, kThreads, 0, L.stream, j, w);
