@@ -193,7 +193,11 @@ constexpr int kSvWarps = 8;            // warps, hence units, per k_sieve CTA
 // A batch's larger sets: units of kSvBatchLen points, kSvBatchUnits per set at
 // most (larger sets take the pipeline), tables of kSvBatchRows bands.
 constexpr int kSvBatchLen = 2048, kSvBatchUnits = 1024, kSvBatchRows = 256;
-constexpr int kSvRows = 256, kSvRefineRows = 512;   // bands per axis of a single set's tables
+// Bands per axis of a single set's tables: of the sample's polygon, and of
+// k_refine's, which has the listed points' own (512 in both: 20M square / disk
+// 144 / 157 us a call, 5M Gaussian 78; 256 and 512: 141 / 152, 73; 256 and
+// 1024: 3 us more on the square, 6 less on a 2M annulus).
+constexpr int kSvRows = 256, kSvRefineRows = 512;
 // Device side of it: the maps of the bands (of Y: s[0] Y + o[0], of X: s[1] X +
 // o[1]), whether the sieve runs (mode) and the number of listed points.
 struct alignas(16) SieveHdr {

@@ -6,10 +6,10 @@
 // regions before the classification) and its dominance tables leave many
 // points where the hull is round (20M disk: 60,000).  Here
 //   k_table    one cluster per set reduces a spread sample to a polygon and
-//              writes a table of horizontal bands with the polygon's left and
-//              right chord in each;
-//   k_sieve    reads every point once and lists the indices of those not
-//              certainly inside their band's chords, in index order;
+//              writes tables of bands, of Y with the polygon's left and right
+//              chord in each and of X with its lower and upper one;
+//   k_sieve    reads every point once and lists the indices of those that
+//              neither axis' chords certainly hold, in index order;
 //   k_refine   one cluster per set gathers the listed points; where they are
 //              many it builds the polygon of the listed points themselves and
 //              lists only those outside it;
@@ -26,7 +26,8 @@
 // that fail the float64 domain check are always listed, so the check reports
 // the same status.
 //
-// The bands.  Everything is computed on FP32 views (float64 truncated, int32
+// The bands (of Y; those of X are the same with the axes exchanged, and hold
+// where the polygon runs level).  Everything is computed on FP32 views (float64 truncated, int32
 // rounded: within 2 u |v| of v, u = 2^-24; magnitudes below 2^-126 within
 // 2^-126, covered because the maxima xm, ym of |X|, |Y| over the sample are at
 // least 2^-100).  The sample's left and right polylines run from its lowest to
@@ -401,7 +402,13 @@ __device__ __forceinline__ SieveHdr fresh_hdr(const SieveHdr* h) {
   return SieveHdr{{v.x, v.y}, {v.z, v.w}, 0u, 0u};
 }
 
-// Table of each set from a sample spread over it in runs of 32 points.
+// Tables of each set from a sample spread over it in runs of 32 points, at most
+// n / 8 of them.  What bounds it is a chain of dependent steps: of 26 us on 20M
+// float64 points, 4 are the sample's loads, 3 its extremes, 7 the bands' minima,
+// 1 the merge, 6 the peeling, 3 the chords and 2 the check at the end.  16 CTAs
+// with 8 points per thread (8 with 16: 46 us); 131,072 points leave 23,600 of a
+// 20M disk and 5,100 of a square; a sixteenth of the set instead of an eighth
+// changed nothing below 2M points.
 template <int DT, int R, int CL, int T, int NI>
 __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   griddep_enter();
@@ -451,7 +458,13 @@ constexpr int kSvThreads = kSvWarps * 32;
 template <int DT>
 constexpr int sv_items() { return DT == DT_F64 ? 4 : 8; }
 
-// One warp per unit of consecutive points.
+// One warp per unit of consecutive points, two batches of loads in registers.
+// float64 is bound by memory: 20M points in 55 us (5.8 TB/s), 46 behind k_table,
+// which lets it prefetch 64 MB into L2 meanwhile (96 and 128 MB: the same).
+// The 8-byte formats are bound by latency and the scattered reads of the table
+// (11 shared wavefronts per 32 points): 20M float32 points in 44 us.  Slower: a
+// four-stage cp.async ring per warp at 24 warps per SM (59 / 51 us), a box test
+// before the table (149 against 143 us a call on the 20M square).
 template <int DT, int R>
 __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
   constexpr int U = sv_items<DT>();
@@ -547,7 +560,10 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
 }
 
 // Listed points of the set gathered in index order; outside the polygon of
-// the listed points themselves where there are more than kPlain.
+// the listed points themselves where there are more than kPlain (20M disk:
+// 23,600 to 2,300 in 30 us, the steps of k_table again; k_set on the longer list
+// takes more than it saves -- with kPlain at 6144 the 20M square, 5,100 listed,
+// went from 143 to 179 us).
 template <int DT, int R, int CL>
 __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
   griddep_enter();
@@ -667,6 +683,40 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
 constexpr int kSvCluster = 16;                     // CTAs per cluster (more than 8: opt-in)
 constexpr int64_t kSvPrefetch = int64_t(64) << 20;  // bytes k_sieve prefetches while k_table runs
 
+// Clusters of kernel fn (attributes set) that fit the device at once.
+int clusters_resident(const void* fn, size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = kSvCluster;
+  cfg.blockDim = kTabThreads;
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kSvCluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+  return n;
+}
+
+// Sets the single-set kernels' attributes; whether their clusters can run here.
+template <int DT>
+bool sieve_fits() {
+  constexpr size_t sm = sizeof(TabSmem<kSvRows, kTabThreads>), smr = sizeof(TabSmem<kSvRefineRows, kTabThreads>);
+  static const bool ok = [] {
+    auto* t = k_table<DT, kSvRows, kSvCluster, kTabThreads, kTabItems>;
+    auto* r = k_refine<DT, kSvRefineRows, kSvCluster>;
+    cudaFuncSetAttribute(t, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(t, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
+    cudaFuncSetAttribute(r, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return clusters_resident((const void*)t, sm) > 0 && clusters_resident((const void*)r, smr) > 0;
+  }();
+  return ok;
+}
+
 template <int DT>
 int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
   constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
@@ -682,12 +732,6 @@ int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
     }
     return 1;
   }
-  static bool once = [] {
-    cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_table<DT, R, CL, T, kTabItems>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return true;
-  }();
-  (void)once;
   launch_pdl_cluster(k_table<DT, R, CL, T, kTabItems>, CL, T, CL, sm, st, j, w);
   return 1;
 }
@@ -695,8 +739,8 @@ int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
 template <int DT>
 int launch_sieve_t(const Job& j, const Ws& w, cudaStream_t st) {
   static_assert(kSvRows == kSvBatchRows, "one k_sieve for both");
-  launch_pdl(k_sieve<DT, kSvRows>, j.sv_sets ? j.sv_nctas : (j.sieve.nunit + kSvWarps - 1) / kSvWarps, kSvThreads, 0, st,
-             j, w);
+  const int grid = j.sv_sets ? j.sv_nctas : (j.sieve.nunit + kSvWarps - 1) / kSvWarps;
+  launch_pdl(k_sieve<DT, kSvRows>, grid, kSvThreads, 0, st, j, w);
   return 1;
 }
 
@@ -704,12 +748,6 @@ template <int DT>
 int launch_refine_t(const Job& j, const Ws& w, cudaStream_t st) {
   constexpr int CL = kSvCluster, R = kSvRefineRows;
   constexpr size_t sm = sizeof(TabSmem<R, kTabThreads>);
-  static bool once = [] {
-    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_refine<DT, R, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return true;
-  }();
-  (void)once;
   launch_pdl_cluster(k_refine<DT, R, CL>, CL, kTabThreads, CL, sm, st, j, w);
   return 1;
 }
@@ -720,6 +758,7 @@ SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms) {
   const int64_t step = 32 * (dtype == DT_F64 ? sv_items<DT_F64>() : sv_items<DT_I32>());
   const int64_t most = std::min<int64_t>((int64_t)sms * 4 * kSvWarps, kSvMaxUnits);
   SieveSet s{};
+  if (!(dtype == DT_F64 ? sieve_fits<DT_F64>() : dtype == DT_F32 ? sieve_fits<DT_F32>() : sieve_fits<DT_I32>())) return s;
   s.off = off;
   s.n = n;
   s.len = ((n + most - 1) / most + step - 1) / step * step;
