@@ -34,6 +34,11 @@ template <>
 struct SetClass<2> { static constexpr int CAP = 4096, T = 256, NB = 512; };
 template <>
 struct SetClass<3> { static constexpr int CAP = 16384, T = 512, NB = 1280; };
+// The sieve's lists of a single set: one CTA per SM in any case, so more warps
+// cost only their barriers (512 -> 1024 threads, us per call: 2M annulus 147 ->
+// 135, 48,007 degenerate points 143 -> 127, 1M int32 square 56 -> 58).
+template <>
+struct SetClass<4> { static constexpr int CAP = 16384, T = 1024, NB = 1280; };
 static_assert(SetClass<kSetClasses - 1>::CAP == kSetMax + 1, "the largest class ends at kSetMax");
 
 // Point c of the set, and the index it is reported as: its own, or that of the
@@ -440,7 +445,7 @@ int launch_set(const Job& j, int cls, const SetItem* items, int count, bool besi
 template <int DT>
 static int launch_set_list_t(const Job& l, const Ws& w, cudaStream_t st) {
   if (!l.sv_sets) {
-    launch_set_c<DT, 3, SET_LIST>(l, nullptr, w, 4, false, st);
+    launch_set_c<DT, 4, SET_LIST>(l, nullptr, w, 4, false, st);
     return 1;
   }
   launch_set_c<DT, 2, SET_BATCH>(l, nullptr, w, l.nsets, false, st);

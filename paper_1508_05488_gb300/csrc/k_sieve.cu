@@ -58,6 +58,8 @@ constexpr int kTabBatchThreads = 256;               // of k_table on a batch's s
                                                     // sets per SM (512 threads, two: 37 us for 409 sets, 30 so)
 constexpr int kTabItems = 8, kTabBatchItems = 16;   // points per thread at most
 constexpr int kPeel = 40;                           // peeling rounds at most
+constexpr int64_t kLeast = 8;                       // a set of which more than this share and more than kSetMax
+                                                    // points are left is refused
 constexpr uint32_t kPlain = 2048;                   // lists up to this size go to k_set as they are
 
 template <int DT>
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   }
   if (rank == 0 && tid == 0) {
     const int64_t left = ok ? (int64_t)m.cnt * sd.n / (min(groups, (int64_t)CL * W) * 32) : sd.n;
-    hdr->mode = ok && left <= sd.cap ? 1u : 0u;
+    hdr->mode = ok && left <= min(sd.cap, max(sd.n / kLeast, (int64_t)kSetMax)) ? 1u : 0u;
   }
 }
 
@@ -722,14 +724,12 @@ int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
   constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
   constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>);
   if (j.sv_sets) {
-    if constexpr (DT != DT_F32) {            // no batches of float32 vectors
-      static bool once = [] {
-        cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
-        return true;
-      }();
-      (void)once;
-      launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
-    }
+    static bool once = [] {
+      cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
+      return true;
+    }();
+    (void)once;
+    launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
     return 1;
   }
   launch_pdl_cluster(k_table<DT, R, CL, T, kTabItems>, CL, T, CL, sm, st, j, w);
