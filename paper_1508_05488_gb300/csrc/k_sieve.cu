@@ -411,6 +411,10 @@ __device__ __forceinline__ SieveHdr fresh_hdr(const SieveHdr* h) {
 // with 8 points per thread (8 with 16: 46 us); 131,072 points leave 23,600 of a
 // 20M disk and 5,100 of a square; a sixteenth of the set instead of an eighth
 // changed nothing below 2M points.
+// A set of which the check finds too much left is refused: points on a circle,
+// all left, take 114 / 211 / 258 / 308 / 383 us at 13, 20, 32, 48 and 65 thousand
+// (136 / 235 / 281 / 337 / 414 when k_refine found out); a fifth left (the
+// degenerate kind) is listed up to kSetMax points.
 template <int DT, int R, int CL, int T, int NI>
 __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   griddep_enter();
