@@ -3,7 +3,9 @@
 //
 // Pipeline (Sec. 2.1, steps 1-7), every stage a kernel, every set of points a
 // "set" (a single hull is a batch of one).  Small sets are computed whole by
-// one CTA each (k_set.cu, hull_block.cuh); the others take the pipeline:
+// one CTA each (k_set.cu, hull_block.cuh); larger ones go through one pass that
+// drops what a sample's polygon covers (k_sieve.cu); what that refuses, and the
+// stage extraction, takes the pipeline:
 //   a1  k_extremes      four lexicographic extremes + edge set-up (step 1)
 //       k_stairs        dominance tables and box from a sample of each set;
 //                       its sample pass runs during a1's tail
