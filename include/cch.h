@@ -37,6 +37,15 @@
  * serialised by the stream; calls on different streams use different
  * workspaces and may overlap on the device.
  *
+ * GRAPHS: cch_hull, cch_hull_f32soa and cch_hull_noalloc may be captured into
+ * a CUDA graph, which may then be launched any number of times on whatever the
+ * points' buffer holds, beside plain calls on the stream of the capture but
+ * not at the same time.  Make a plain call of the same size on that stream
+ * first where the capture forbids allocation.  The graph uses that stream's
+ * workspace: it must not be launched after cch_release_workspace().
+ * cch_hull_batched reads tables from host memory that belongs to the library
+ * and must not be captured.
+ *
  * ERRORS: the return value reports what the host can see before launching
  * (bad arguments, allocation or launch failure) as a negative CCH_ERR_*
  * code; nothing is launched then.  Errors found on the device (non-finite or

@@ -94,7 +94,10 @@ struct Workspace {
   char* dev = nullptr;
   size_t bytes = 0;
   Dims cap{};
-  uint32_t epoch = 0;
+  uint32_t epoch = 0;                // of the last plain call
+  bool uncleared = false;            // allocated while a graph was captured: cleared by its runs only
+  bool captured = false;             // a graph holds `dev`
+  std::vector<char*> retired;        // earlier buffers that a graph holds
   char* host_tab = nullptr;          // pinned staging of a batch's tables
   char* dev_tab = nullptr;           // their device copy
   size_t tab_bytes = 0;              // size of both
@@ -150,8 +153,10 @@ bool fits(const Dims& c, const Dims& d) {
   return d.N <= c.N && d.nsets <= c.nsets && d.nchunk1 <= c.nchunk1 && d.ntile2 <= c.ntile2;
 }
 
-// Grow the workspace `ws` of `stream` to dims `d`.  Called with g_mu held.
-int acquire(cudaStream_t stream, const Dims& d, Workspace* ws) {
+// Grow the workspace `ws` of `stream` to dims `d`; `graph`: the stream is being
+// captured.  A buffer that a graph holds stays allocated until the workspace is
+// released: the graph may be launched again.  Called with g_mu held.
+int acquire(cudaStream_t stream, const Dims& d, Workspace* ws, bool graph) {
   if (!ws->dev || !fits(ws->cap, d)) {
     Dims c = d;
     if (ws->dev) {   // grow by at least 1.5x to amortise
@@ -161,8 +166,10 @@ int acquire(cudaStream_t stream, const Dims& d, Workspace* ws) {
       c.ntile2 = std::max(d.ntile2, ws->cap.ntile2);
       c = make_dims(c.N, c.nsets, c.nchunk1, (int32_t)std::max<int64_t>(c.ntile2, c.N / kClsMinTile + c.nsets + 1));
       if (cudaStreamSynchronize(stream) != cudaSuccess) return CCH_ERR_CUDA;
-      cudaFree(ws->dev);
+      if (ws->captured) ws->retired.push_back(ws->dev);
+      else cudaFree(ws->dev);
       ws->dev = nullptr;
+      ws->captured = false;
     }
     Layout L = layout(c, nullptr);
     if (cudaMalloc(&ws->dev, L.total) != cudaSuccess) {
@@ -182,7 +189,12 @@ int acquire(cudaStream_t stream, const Dims& d, Workspace* ws) {
     ws->bytes = L.total;
     ws->cap = c;
     ws->epoch = 0;
+    ws->uncleared = graph;
+  } else if (ws->uncleared && !graph) {
+    if (cudaMemsetAsync(ws->dev, 0, ws->bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
+    ws->uncleared = false;
   }
+  ws->captured |= graph;
   return CCH_OK;
 }
 
@@ -288,14 +300,19 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
       return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
     }
   }
-  int st = acquire(stream, d, ws);
+  const bool graph = capturing(stream);
+  int st = acquire(stream, d, ws, graph);
   if (st != CCH_OK) return st;
   Layout L = layout(ws->cap, ws->dev);
-  if (++ws->epoch > 0xFFFu) {
-    if (cudaMemsetAsync(ws->dev + L.status_off, 0, L.status_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
-    ws->epoch = 1;
+  if (graph) {
+    j.epoch = kEpochGraph;
+  } else {
+    if (++ws->epoch > kEpochLast) {
+      if (cudaMemsetAsync(ws->dev + L.status_off, 0, L.status_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
+      ws->epoch = 1;
+    }
+    j.epoch = ws->epoch;
   }
-  j.epoch = ws->epoch;
   if (cudaMemsetAsync(ws->dev, 0, L.ctl_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
   if (stages) { j.r1_idx = stages->r1_idx; j.r1_region = stages->r1_region; }
   ProfRec rec{};
@@ -325,6 +342,9 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
     nk += launch_set_list(j, L.w, stream);
     mark_sv(4);
   }
+  // (on the pipeline's stream: a sieved run's lists do not wait for it)
+  if (graph && cudaMemsetAsync(ws->dev + L.status_off, 0, L.status_bytes, side ? ws->side : stream) != cudaSuccess)
+    return CCH_ERR_CUDA;
   Launch La{side ? ws->side : stream, grid_cap(), j.tune.cls_per_sm * sm_count()};
   // event k marks the start of stage k (and the end of stage k - 1)
   auto mark = [&](int k) {
@@ -689,6 +709,7 @@ void cch_release_workspace(void) {
   for (auto& kv : g_ws) {
     Workspace* ws = kv.second;
     if (ws->dev) cudaFree(ws->dev);
+    for (char* p : ws->retired) cudaFree(p);
     if (ws->host_tab) cudaFreeHost(ws->host_tab);
     if (ws->dev_tab) cudaFree(ws->dev_tab);
     if (ws->tab_done) cudaEventDestroy(ws->tab_done);

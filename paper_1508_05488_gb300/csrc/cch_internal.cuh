@@ -220,7 +220,7 @@ struct Job {
   int32_t nchunk3;      // total stairs chunks
   int32_t nchunkP;      // total survivor-count chunks
   int64_t chunk1_len;   // a1 chunk length (points), multiple of 256
-  uint32_t epoch;       // look-back flag epoch of this call (1..0xFFFF)
+  uint32_t epoch;       // look-back epoch of this call (kEpochLast, kEpochGraph)
   uint32_t opts;        // OPT_* bits
   uint32_t fast_sort;   // a single set whose multi-block sort may go by quantised keys
   Tune tune;            // run-time choices (the same results with any valid choice)
@@ -720,9 +720,9 @@ __device__ __forceinline__ void st_rel_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
-// Packed look-back word: [epoch:16 | kind:16 | value:32]; kind 1 = tile
-// aggregate, 2 = inclusive prefix.  A word from an older call or pass has a
-// different epoch/kind tag and reads as "not ready".
+// Packed look-back word: [epoch:12 | phase:4 | kind:16 | value:32]; kind 1 =
+// tile aggregate, 2 = inclusive prefix.  A word from an older call or pass has
+// a different epoch/phase tag and reads as "not ready".
 __device__ __forceinline__ uint64_t lb_pack(uint32_t tag, uint32_t kind, uint32_t v) {
   return ((uint64_t)((tag << 16) | kind) << 32) | v;
 }
@@ -1028,6 +1028,20 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args... args) {
   return launch_pdl_cluster(kernel, grid, block, 1, smem, st, args...);
+}
+
+// Look-back epochs.  A plain call takes the next of 1..kEpochLast, and the
+// words are cleared when they start again.  A call that is captured into a
+// graph runs many times with the epoch it was captured with: its graph clears
+// the words on every run, and its epoch is one that no plain call takes, so the
+// words it leaves are not ready to any of them.
+constexpr uint32_t kEpochLast = 0xFFEu, kEpochGraph = 0xFFFu;
+
+// Whether the stream is being captured into a graph.
+inline bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { cudaGetLastError(); return false; }
+  return s == cudaStreamCaptureStatusActive;
 }
 
 // ------------------------------------------------------------ launchers

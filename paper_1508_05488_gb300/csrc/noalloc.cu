@@ -19,9 +19,11 @@
 //     last call's contents.  The array has one fixed layout, sized for the
 //     largest call, so every buffer sits at the same place in every call.
 //     The per-call control words are cleared by each call.  Look-back words
-//     carry the call's epoch (1..4095) and read as "not ready" in any other
+//     carry the call's epoch (1..4094) and read as "not ready" in any other
 //     call; when the epoch wraps, the whole look-back region is cleared, so
-//     no word of an earlier cycle can be taken for one of this call;
+//     no word of an earlier cycle can be taken for one of this call.  A
+//     captured call clears the region on every run of its graph and has an
+//     epoch of its own;
 //   * calls whose work overlaps on the GPU (different streams, no ordering
 //     between them) race on the shared array and give wrong results: order
 //     them (one stream, or events);
@@ -163,11 +165,13 @@ extern "C" int cch_hull_noalloc(const void* points, int64_t n, int dtype, int32_
   const size_t need = na_layout(g_na_ptr[dev], w, ctl_bytes, status_off, status_bytes);
   if (need > kNoAllocBytes) return CCH_ERR_RANGE;
 
-  if (++g_na_epoch[dev] > 0xFFFu) {
+  const bool graph = capturing(st);
+  const bool wrap = !graph && ++g_na_epoch[dev] > kEpochLast;
+  if (graph || wrap) {
     if (cudaMemsetAsync(g_na_ptr[dev] + status_off, 0, status_bytes, st) != cudaSuccess) return CCH_ERR_CUDA;
-    g_na_epoch[dev] = 1;
+    if (wrap) g_na_epoch[dev] = 1;
   }
-  j.epoch = g_na_epoch[dev];
+  j.epoch = graph ? kEpochGraph : g_na_epoch[dev];
   if (cudaMemsetAsync(g_na_ptr[dev], 0, ctl_bytes, st) != cudaSuccess) return CCH_ERR_CUDA;
 
   Launch L{st, sms * 4, 2 * sms};
