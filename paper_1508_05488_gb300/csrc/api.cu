@@ -292,6 +292,12 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   if (!slot) slot = new Workspace();
   Workspace* ws = slot;
   int nk = 0;
+  const bool graph = capturing(stream);
+  // every allocation first: a call that fails for want of memory launches nothing
+  if (!batch || !batch->sets.empty()) {
+    const int st = acquire(stream, d, ws, graph);
+    if (st != CCH_OK) return st;
+  }
   if (batch) {
     const int st = start_batch(j, *batch, ws, stream, &nk);
     if (st != CCH_OK) return st;
@@ -300,9 +306,6 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
       return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
     }
   }
-  const bool graph = capturing(stream);
-  int st = acquire(stream, d, ws, graph);
-  if (st != CCH_OK) return st;
   Layout L = layout(ws->cap, ws->dev);
   if (graph) {
     j.epoch = kEpochGraph;
