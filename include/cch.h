@@ -43,8 +43,9 @@
  * not at the same time.  Make a plain call of the same size on that stream
  * first where the capture forbids allocation.  The graph uses that stream's
  * workspace: it must not be launched after cch_release_workspace().
- * cch_hull_batched reads tables from host memory that belongs to the library
- * and must not be captured.
+ * cch_hull_batched may be captured in a mode that allows allocation (its set
+ * tables get staging of their own, kept until cch_release_workspace()); its
+ * offsets are those of the capture.
  *
  * ERRORS: the return value reports what the host can see before launching
  * (bad arguments, allocation or launch failure) as a negative CCH_ERR_*

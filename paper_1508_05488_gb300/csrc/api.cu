@@ -97,7 +97,8 @@ struct Workspace {
   uint32_t epoch = 0;                // of the last plain call
   bool uncleared = false;            // allocated while a graph was captured: cleared by its runs only
   bool captured = false;             // a graph holds `dev`
-  std::vector<char*> retired;        // earlier buffers that a graph holds
+  std::vector<char*> retired;        // earlier buffers and tables that a graph holds
+  std::vector<char*> retired_host;   // its tables' staging
   char* host_tab = nullptr;          // pinned staging of a batch's tables
   char* dev_tab = nullptr;           // their device copy
   size_t tab_bytes = 0;              // size of both
@@ -219,16 +220,22 @@ struct Batch {
   std::vector<SetItem> items[kSetClasses];
 };
 
-// Copy a batch's tables (small sets by class, then the larger sets) to the
-// device, and launch k_set on the small ones.  Called with g_mu held; returns
-// a status, the kernels launched are added to *nk.
-int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int* nk) {
-  size_t ibytes = 0;
-  for (const auto& v : b.items) ibytes += sizeof(SetItem) * v.size();
-  const size_t sets_off = (ibytes + 63) / 64 * 64;
-  const size_t sv_off = sets_off + (sizeof(SetDesc) * b.sets.size() + 63) / 64 * 64;
-  const size_t cta_off = sv_off + sizeof(SieveSet) * b.sieve.size();
-  const size_t bytes = cta_off + sizeof(int32_t) * b.cta.size();
+// Staging for a batch's tables: the workspace's, free of the last call's copy.
+// A graph copies from the staging on every run, so a captured call has its own,
+// kept until the workspace is released (an event recorded under a capture could
+// not be waited for, and a later call would change the graph's tables).
+int stage_tables(Workspace* ws, size_t bytes, cudaStream_t stream, bool graph, char*& host, char*& dev) {
+  if (graph) {
+    host = dev = nullptr;
+    if (cudaMallocHost(&host, bytes) != cudaSuccess || cudaMalloc(&dev, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      if (host) cudaFreeHost(host);
+      return CCH_ERR_NOMEM;
+    }
+    ws->retired_host.push_back(host);
+    ws->retired.push_back(dev);
+    return CCH_OK;
+  }
   if (!ws->tab_done && cudaEventCreateWithFlags(&ws->tab_done, cudaEventDisableTiming) != cudaSuccess) return CCH_ERR_CUDA;
   if (cudaEventSynchronize(ws->tab_done) != cudaSuccess) return CCH_ERR_CUDA;
   if (ws->tab_bytes < bytes) {
@@ -246,19 +253,38 @@ int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int*
     }
     ws->tab_bytes = cap;
   }
+  host = ws->host_tab;
+  dev = ws->dev_tab;
+  return CCH_OK;
+}
+
+// Copy a batch's tables (small sets by class, then the larger sets) to the
+// device, and launch k_set on the small ones; `graph`: the stream is being
+// captured.  Called with g_mu held; returns a status, the kernels launched are
+// added to *nk.
+int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool graph, int* nk) {
+  size_t ibytes = 0;
+  for (const auto& v : b.items) ibytes += sizeof(SetItem) * v.size();
+  const size_t sets_off = (ibytes + 63) / 64 * 64;
+  const size_t sv_off = sets_off + (sizeof(SetDesc) * b.sets.size() + 63) / 64 * 64;
+  const size_t cta_off = sv_off + sizeof(SieveSet) * b.sieve.size();
+  const size_t bytes = cta_off + sizeof(int32_t) * b.cta.size();
+  char *host, *dev;
+  const int st = stage_tables(ws, bytes, stream, graph, host, dev);
+  if (st != CCH_OK) return st;
   size_t o = 0;
   for (const auto& v : b.items) {
-    if (!v.empty()) memcpy(ws->host_tab + o, v.data(), sizeof(SetItem) * v.size());
+    if (!v.empty()) memcpy(host + o, v.data(), sizeof(SetItem) * v.size());
     o += sizeof(SetItem) * v.size();
   }
   if (!b.sets.empty()) {
-    memcpy(ws->host_tab + sets_off, b.sets.data(), sizeof(SetDesc) * b.sets.size());
-    memcpy(ws->host_tab + sv_off, b.sieve.data(), sizeof(SieveSet) * b.sieve.size());
-    if (!b.cta.empty()) memcpy(ws->host_tab + cta_off, b.cta.data(), sizeof(int32_t) * b.cta.size());
+    memcpy(host + sets_off, b.sets.data(), sizeof(SetDesc) * b.sets.size());
+    memcpy(host + sv_off, b.sieve.data(), sizeof(SieveSet) * b.sieve.size());
+    if (!b.cta.empty()) memcpy(host + cta_off, b.cta.data(), sizeof(int32_t) * b.cta.size());
   }
-  if (cudaMemcpyAsync(ws->dev_tab, ws->host_tab, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
-  if (cudaEventRecord(ws->tab_done, stream) != cudaSuccess) return CCH_ERR_CUDA;
-  const SetItem* items = reinterpret_cast<const SetItem*>(ws->dev_tab);
+  if (cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
+  if (!graph && cudaEventRecord(ws->tab_done, stream) != cudaSuccess) return CCH_ERR_CUDA;
+  const SetItem* items = reinterpret_cast<const SetItem*>(dev);
   o = 0;
   for (int c = 0; c < kSetClasses; c++) o += b.items[c].size();
   // the largest sets first; a class starts beside the one before it where that
@@ -274,11 +300,11 @@ int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, int*
     *nk += launch_set(j, c, items + o, (int)b.items[c].size(), beside, stream);
   }
   if (!b.cta.empty()) {
-    j.sv_sets = reinterpret_cast<const SieveSet*>(ws->dev_tab + sv_off);
-    j.sv_cta = reinterpret_cast<const int32_t*>(ws->dev_tab + cta_off);
+    j.sv_sets = reinterpret_cast<const SieveSet*>(dev + sv_off);
+    j.sv_cta = reinterpret_cast<const int32_t*>(dev + cta_off);
     j.sv_nctas = (int32_t)b.cta.size();
   }
-  j.sets = reinterpret_cast<const SetDesc*>(ws->dev_tab + sets_off);
+  j.sets = reinterpret_cast<const SetDesc*>(dev + sets_off);
   return CCH_OK;
 }
 
@@ -299,7 +325,7 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
     if (st != CCH_OK) return st;
   }
   if (batch) {
-    const int st = start_batch(j, *batch, ws, stream, &nk);
+    const int st = start_batch(j, *batch, ws, stream, graph, &nk);
     if (st != CCH_OK) return st;
     if (batch->sets.empty()) {
       g_launches += (uint64_t)nk;
@@ -713,6 +739,7 @@ void cch_release_workspace(void) {
     Workspace* ws = kv.second;
     if (ws->dev) cudaFree(ws->dev);
     for (char* p : ws->retired) cudaFree(p);
+    for (char* p : ws->retired_host) cudaFreeHost(p);
     if (ws->host_tab) cudaFreeHost(ws->host_tab);
     if (ws->dev_tab) cudaFree(ws->dev_tab);
     if (ws->tab_done) cudaEventDestroy(ws->tab_done);

@@ -118,3 +118,52 @@ def test_replay_after_the_workspace_has_grown():
             got = cch.hull(torch.from_numpy(big).to(DEV))
         assert np.array_equal(got.cpu().numpy(), oracle.hull(big))
         c.replay(inputs.circle_f64(60_001, seed))
+
+
+def batch_sets(sizes, seed):
+    gens = [inputs.disk_f64, inputs.circle_f64, inputs.square_f64]
+    return [gens[k % 3](n, seed + k) for k, n in enumerate(sizes)]
+
+
+def test_captured_batch_between_plain_batches():
+    """A batch's graph keeps its own tables; a plain batch of other sizes on the stream is not in its way, nor
+    is an earlier capture that the mode refused."""
+    sizes, other = [500, 30_001, 1500, 9000, 20_011, 70_003, 40_000], [700, 25_000, 16_000, 3000]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    n = int(off[-1])
+    s = torch.cuda.Stream()
+    pts = torch.zeros((n, 2), dtype=torch.float64, device=DEV)
+    idx = torch.zeros(n, dtype=torch.int32, device=DEV)
+    cnt = torch.zeros(len(sizes), dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+
+    def check(sets):
+        torch.cuda.synchronize()
+        for k, p in enumerate(sets):
+            a = int(off[k])
+            assert np.array_equal(idx[a:a + int(cnt[k])].cpu().numpy(), oracle.hull(p)), k
+
+    def plain():
+        sets = batch_sets(other, 50)
+        with torch.cuda.stream(s):
+            got = cch.hull_batched(torch.from_numpy(np.concatenate(sets)).to(DEV), np.concatenate([[0], np.cumsum(other)]))
+        for h, p in zip(got, sets):
+            assert np.array_equal(h.cpu().numpy(), oracle.hull(p))
+
+    with torch.cuda.stream(s):
+        cch.hull_batched_async(pts, off, idx, cnt)
+    s.synchronize()
+    with pytest.raises(Exception):
+        with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=s, capture_error_mode="global"):
+            cch.hull_batched_async(pts, off, idx, cnt)
+    plain()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+        cch.hull_batched_async(pts, off, idx, cnt)
+    for seed in (1, 20, 40):
+        plain()
+        sets = batch_sets(sizes, seed)
+        pts.copy_(torch.from_numpy(np.concatenate(sets)))
+        torch.cuda.synchronize()
+        g.replay()
+        check(sets)
