@@ -155,6 +155,13 @@ def _check_points(points):
         raise ValueError("points must be a contiguous [n, 2] tensor")
 
 
+def _on(stream):
+    """Context in which tensors are allocated and read on `stream` (default: current stream)."""
+    import contextlib
+    import torch
+    return contextlib.nullcontext() if stream is None else torch.cuda.stream(stream)
+
+
 def hull_async(points, out_idx=None, out_count=None, stream=None):
     """Enqueue one hull on `stream` (default: current stream).
 
@@ -178,8 +185,9 @@ def hull_async(points, out_idx=None, out_count=None, stream=None):
 def hull(points, stream=None):
     """Hull vertex indices (int32 CUDA tensor, CCW from the lexicographic
     minimum).  Synchronises the stream to read the count."""
-    out_idx, out_count = hull_async(points, stream=stream)
-    h = int(out_count.item())
+    with _on(stream):
+        out_idx, out_count = hull_async(points, stream=stream)
+        h = int(out_count.item())
     if h < 0:
         raise CchError(h, "cch_hull (device)")
     return out_idx[:h]
@@ -211,8 +219,9 @@ def hull_f32soa_async(x, y, out_idx=None, out_count=None, stream=None):
 
 def hull_f32soa(x, y, stream=None):
     """Hull vertex indices of float32 SoA points (synchronises)."""
-    out_idx, out_count = hull_f32soa_async(x, y, stream=stream)
-    h = int(out_count.item())
+    with _on(stream):
+        out_idx, out_count = hull_f32soa_async(x, y, stream=stream)
+        h = int(out_count.item())
     if h < 0:
         raise CchError(h, "cch_hull_f32soa (device)")
     return out_idx[:h]
@@ -241,8 +250,9 @@ def hull_batched_async(points, offsets, out_idx=None, out_counts=None, stream=No
 
 def hull_batched(points, offsets, stream=None):
     """List of per-set hull index tensors (synchronises)."""
-    out_idx, out_counts = hull_batched_async(points, offsets, stream=stream)
-    counts = out_counts.cpu().numpy()
+    with _on(stream):
+        out_idx, out_counts = hull_batched_async(points, offsets, stream=stream)
+        counts = out_counts.cpu().numpy()
     res = []
     for s in range(len(offsets) - 1):
         h = int(counts[s])
