@@ -19,8 +19,9 @@ namespace cch {
 constexpr int kBlkMax = 16384;          // candidate numbers are below it (14 bits); a block takes fewer than
                                         // CAP <= kBlkMax points, so no entry is 0xFFFF, the sort's padding
 // Ranking a bucket compares its members pair by pair, sum(occ^2) comparisons in
-// all; above kBlkPairs per kept candidate (many equal keys) a bitonic sort of
-// log2(m)^2 / 2 passes is the cheaper one.
+// all; above kBlkPairs per kept candidate (many equal keys) the candidates behind
+// their bucket's best one go first, and a bitonic sort of log2(m)^2 / 2 passes
+// takes the rest.
 constexpr uint32_t kBlkPairs = 128;
 constexpr uint16_t kPin = 0x8000u;      // polygon entry that is one of E1..E4
 
@@ -480,7 +481,7 @@ __device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src) {
     blk_append(m.b, &m.n[1], keep, e);
   }
   __syncthreads();
-  const uint32_t m2 = m.n[1];
+  uint32_t m2 = m.n[1];
   if (m2 != 0) {                              // uniform
     // bucket starts
     {
@@ -520,8 +521,49 @@ __device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src) {
         m.b[st + rank] = (uint16_t)e;
       }
     } else {
-      // crowded buckets (equal or nearly equal keys): bitonic sort by
-      // (region, key, c); the pad entries 0xFFFF sort last
+      // Crowded buckets (equal or nearly equal keys: a flat side, copies).  With
+      // f the bucket's smallest by (SPA value, key, c), another candidate e
+      // whose key is not below f's is no vertex: the line from f through e
+      // (right of f or level, above it or level, in region 1's terms) meets the
+      // segment E_r E_{r+1} behind e, which is outside it; a copy of f has a
+      // larger index.  Then a bitonic sort of what is left by (region, key, c),
+      // the pad entries 0xFFFF last.  (2M points on an 801 x 801 grid, 10,000
+      // of them listed from its sides: 316 us a call by the sort alone, 155 so.)
+      for (uint32_t t = tid; t < 4 * NB; t += T) m.tab[t] = 0xFFFFFFFFu;
+      __syncthreads();
+      for (uint32_t t = tid; t < m2; t += T) {
+        const uint32_t e = m.b[t];
+        const int r = (int)(e >> 14);
+        const P p = src.pt(e & 0x3FFFu);
+        const uint64_t v = blk_spa<DT>(p, r), k = blk_key<DT>(p, r);
+        uint32_t* best = &m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
+        uint32_t f = *(volatile uint32_t*)best;
+        for (;;) {
+          if (f != 0xFFFFFFFFu) {
+            const P q = src.pt(f & 0x3FFFu);
+            const uint64_t vf = blk_spa<DT>(q, r), kf = blk_key<DT>(q, r);
+            if (vf < v || (vf == v && (kf < k || (kf == k && f < e)))) break;
+          }
+          const uint32_t o = atomicCAS(best, f, e);   // fails only where a better one came
+          if (o == f) break;
+          f = o;
+        }
+      }
+      __syncthreads();
+      for (uint32_t t0 = 0; t0 < m2; t0 += T) {
+        uint32_t e[1] = {0u}, keep = 0;
+        if (t0 + tid < m2) {
+          e[0] = m.b[t0 + tid];
+          const int r = (int)(e[0] >> 14);
+          const P p = src.pt(e[0] & 0x3FFFu);
+          const uint32_t f = m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
+          keep = f == e[0] || blk_key<DT>(p, r) < blk_key<DT>(src.pt(f & 0x3FFFu), r);
+        }
+        blk_append(m.a, &m.n[3], keep, e);
+      }
+      __syncthreads();
+      m2 = m.n[3];
+      for (uint32_t t = tid; t < m2; t += T) m.b[t] = m.a[t];
       uint32_t N2 = 2;
       while (N2 < m2) N2 <<= 1;
       for (uint32_t t = m2 + tid; t < N2; t += T) m.b[t] = 0xFFFFu;
