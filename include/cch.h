@@ -240,7 +240,11 @@ int cch_hull_noalloc(const void *points, int64_t n, int dtype,
  * n / stair_div))), the smallest a1 chunk, and a2's CTAs per SM.  A table
  * keyed by GPU (name, SM count), dtype, single set or batch, and size bucket
  * (floor(log2(points per set)), cch_tune_bucket) holds them; calls without
- * an entry use the defaults.  The table can be filled by hand, by
+ * an entry use the defaults.  (With the default small_max a single float64 or
+ * float32 set takes the multi-block sort, which has fewer passes there, for
+ * regions above 4096 points.)  They
+ * act on the sets that reach the pipeline behind these choices: not on small
+ * sets, nor on larger ones that the one-pass sieve finishes.  The table can be filled by hand, by
  * cch_autotune_batched, or from a JSON cache file. */
 typedef struct cch_tune_params {
   int32_t small_max;     /* 1 .. 16384 */

@@ -428,6 +428,7 @@ Job single_job(const void* points, int64_t n, int dtype, int32_t* out_idx, int32
   j.dtype = dtype;
   j.opts = opts;
   j.tune = tune_for(dtype, n, 1);
+  j.fast_max = j.tune.small_max == kTuneDefault.small_max ? kFastSmallMax : (uint32_t)j.tune.small_max;
   int target = a1_target(dtype);
   int64_t len = (n + target - 1) / std::max(target, 1);
   len = std::max<int64_t>(j.tune.a1_len_min, (len + 1023) / 1024 * 1024);
@@ -496,7 +497,7 @@ int cch_hull(const void* points, int64_t n, int dtype, int32_t* out_idx, int32_t
   if (n <= kSetOne) return run_set(set_job(points, nullptr, n, dtype, out_idx, out_count), (cudaStream_t)stream);
   Job j = single_job(points, n, dtype, out_idx, out_count, 0);
   j.sieve = sieve_set(0, n, dtype, sm_count());
-  j.fast_sort = 1;
+  j.fast_sort = dtype != CCH_I32;
   return run(j, nullptr, (cudaStream_t)stream, nullptr, nullptr);
 }
 

@@ -207,6 +207,13 @@ struct alignas(16) SieveHdr {
   uint32_t mode, n;
 };
 
+// Largest region that the shared-memory sort takes where the multi-block one has
+// four passes, unless small_max is set to another value than its default.  us per
+// call at 16384 / 8192 / 4096 / 2048: float64 circle of 32,001 points 258 / 258 /
+// 181 / 181, of 65,003 384 / 185 / 186 / 186, degenerate set of 100,003 points
+// 210 / 211 / 179 / 179, of 200,003 277 / 193 / 192 / 194.
+constexpr uint32_t kFastSmallMax = 4096;
+
 // Per-call launch description.  A single hull carries its descriptor inline;
 // a batch points at a device array.
 struct Job {
@@ -222,7 +229,8 @@ struct Job {
   int64_t chunk1_len;   // a1 chunk length (points), multiple of 256
   uint32_t epoch;       // look-back epoch of this call (kEpochLast, kEpochGraph)
   uint32_t opts;        // OPT_* bits
-  uint32_t fast_sort;   // a single set whose multi-block sort may go by quantised keys
+  uint32_t fast_sort;   // a single float set whose multi-block sort goes by quantised keys (SF_SMALL), and
+  uint32_t fast_max;    //   the largest region of the shared-memory sort where it does
   Tune tune;            // run-time choices (the same results with any valid choice)
   const SetDesc* sets;  // device array, or nullptr -> use `one`
   SetDesc one;

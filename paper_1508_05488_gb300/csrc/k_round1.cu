@@ -1467,8 +1467,9 @@ __global__ void __launch_bounds__(kThreads) k_gather(Job j, Ws w) {
         if (lc == 0 && part == 0) {
           // the set's first chunk records its region totals and its path
           SetCtl& cs = w.ctl[s];
+          const uint32_t most = j.fast_sort && (cs.flags & SF_SMALL) ? j.fast_max : j.tune.small_max;
           bool big = false;
-          for (int q = 0; q < 4; q++) { cs.cnt[q] = t[q]; big |= t[q] > (uint32_t)j.tune.small_max; }
+          for (int q = 0; q < 4; q++) { cs.cnt[q] = t[q]; big |= t[q] > most; }
           cs.s1 = t[0] + t[1] + t[2] + t[3];
           // the paper's chunked SPA reads the sorted records from global memory
           if ((j.opts & OPT_BLOCKED_SPA) && cs.s1 > 0) big = true;
