@@ -259,10 +259,9 @@ int stage_tables(Workspace* ws, size_t bytes, cudaStream_t stream, bool graph, c
 }
 
 // Copy a batch's tables (small sets by class, then the larger sets) to the
-// device, and launch k_set on the small ones; `graph`: the stream is being
-// captured.  Called with g_mu held; returns a status, the kernels launched are
-// added to *nk.
-int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool graph, int* nk) {
+// device; *items: the small sets'.  `graph`: the stream is being captured.
+// Called with g_mu held.
+int copy_tables(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool graph, const SetItem** items) {
   size_t ibytes = 0;
   for (const auto& v : b.items) ibytes += sizeof(SetItem) * v.size();
   const size_t sets_off = (ibytes + 63) / 64 * 64;
@@ -284,8 +283,24 @@ int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool
   }
   if (cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CCH_ERR_CUDA;
   if (!graph && cudaEventRecord(ws->tab_done, stream) != cudaSuccess) return CCH_ERR_CUDA;
-  const SetItem* items = reinterpret_cast<const SetItem*>(dev);
-  o = 0;
+  *items = reinterpret_cast<const SetItem*>(dev);
+  if (!b.cta.empty()) {
+    j.sv_sets = reinterpret_cast<const SieveSet*>(dev + sv_off);
+    j.sv_cta = reinterpret_cast<const int32_t*>(dev + cta_off);
+    j.sv_nctas = (int32_t)b.cta.size();
+  }
+  j.sets = reinterpret_cast<const SetDesc*>(dev + sets_off);
+  return CCH_OK;
+}
+
+// k_set on a batch's small sets; the number of kernels launched.  Beside larger
+// sets they run on the workspace's stream, launched last: they take the SMs that
+// the others' latency-bound kernels leave (64 float64 sets of up to 2^18 points,
+// most of them small: 163 us one after the other, 127 so; launched first: 129, and
+// 203 against 199 on 64 int32 sets of up to 2^20).
+int launch_small_sets(const Job& j, const Batch& b, const SetItem* items, cudaStream_t stream) {
+  int nk = 0;
+  size_t o = 0;
   for (int c = 0; c < kSetClasses; c++) o += b.items[c].size();
   // the largest sets first; a class starts beside the one before it where that
   // leaves SMs free (1024 int32 sets, 213, 103, 94 and 205 of them small: 285 us
@@ -297,15 +312,9 @@ int start_batch(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool
     o -= b.items[c].size();
     const bool beside = prev != 0 && prev <= 2 * (size_t)sm_count();
     if (!b.items[c].empty()) prev = b.items[c].size();
-    *nk += launch_set(j, c, items + o, (int)b.items[c].size(), beside, stream);
+    nk += launch_set(j, c, items + o, (int)b.items[c].size(), beside, stream);
   }
-  if (!b.cta.empty()) {
-    j.sv_sets = reinterpret_cast<const SieveSet*>(dev + sv_off);
-    j.sv_cta = reinterpret_cast<const int32_t*>(dev + cta_off);
-    j.sv_nctas = (int32_t)b.cta.size();
-  }
-  j.sets = reinterpret_cast<const SetDesc*>(dev + sets_off);
-  return CCH_OK;
+  return nk;
 }
 
 // Launch the whole call: k_set on a batch's small sets, the pipeline on the
@@ -324,9 +333,16 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
     const int st = acquire(stream, d, ws, graph);
     if (st != CCH_OK) return st;
   }
+  const SetItem* items = nullptr;
+  bool small = false;                  // small sets beside larger ones, launched after them
   if (batch) {
-    const int st = start_batch(j, *batch, ws, stream, graph, &nk);
+    const int st = copy_tables(j, *batch, ws, stream, graph, &items);
     if (st != CCH_OK) return st;
+    size_t nsmall = 0;
+    for (const auto& v : batch->items) nsmall += v.size();
+    small = nsmall != 0 && !batch->sets.empty() && ws->join && !g_prof;
+    if (!small) nk += launch_small_sets(j, *batch, items, stream);
+    else if (cudaEventRecord(ws->fork, stream) != cudaSuccess) return CCH_ERR_CUDA;
     if (batch->sets.empty()) {
       g_launches += (uint64_t)nk;
       return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
@@ -394,8 +410,12 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
   mark(6);
   nk += launch_chain(j, L.w, La);
   mark(7);
-  if (side && (cudaEventRecord(ws->join, ws->side) != cudaSuccess ||
-               cudaStreamWaitEvent(stream, ws->join, 0) != cudaSuccess)) return CCH_ERR_CUDA;
+  if (small) {
+    if (cudaStreamWaitEvent(ws->side, ws->fork, 0) != cudaSuccess) return CCH_ERR_CUDA;
+    nk += launch_small_sets(j, *batch, items, ws->side);
+  }
+  if ((side || small) && (cudaEventRecord(ws->join, ws->side) != cudaSuccess ||
+                          cudaStreamWaitEvent(stream, ws->join, 0) != cudaSuccess)) return CCH_ERR_CUDA;
   if (stages) {
     if (j.opts & OPT_BLOCKED_SPA) nk += launch_spa_blocked(j, L.w, stages->spa_idx, stream);
     else { launch_extract_spa(j, L.w, stages->spa_idx, stream); nk++; }
