@@ -307,12 +307,14 @@ int launch_small_sets(const Job& j, const Batch& b, const SetItem* items, cudaSt
   // a call, 343 one class after the other); where it does not, sharing an SM
   // costs both their L1 (4096 float64 sets of 256 to 4096 points: 259 us
   // beside, 224 one after the other)
+  const size_t sms = (size_t)sm_count(), above = b.items[1].size() + b.items[2].size() + b.items[3].size();
   size_t prev = 0;
   for (int c = kSetClasses - 1; c >= 0; c--) {
     o -= b.items[c].size();
-    const bool beside = prev != 0 && prev <= 2 * (size_t)sm_count();
-    if (!b.items[c].empty()) prev = b.items[c].size();
-    nk += launch_set(j, c, items + o, (int)b.items[c].size(), beside, stream);
+    const size_t count = b.items[c].size();
+    const bool beside = prev != 0 && prev <= 2 * sms, split = c > 0 && 4 * above <= sms;
+    if (count) prev = split ? 4 * count : count;
+    nk += launch_set(j, c, items + o, (int)count, split, beside, stream);
   }
   return nk;
 }
@@ -384,7 +386,7 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
     if (side && (cudaEventRecord(ws->fork, stream) != cudaSuccess ||
                  cudaStreamWaitEvent(ws->side, ws->fork, 0) != cudaSuccess)) return CCH_ERR_CUDA;
     mark_sv(3);
-    nk += launch_set_list(j, L.w, stream);
+    nk += launch_set_list(j, L.w, sm_count(), stream);
     mark_sv(4);
   }
   // (on the pipeline's stream: a sieved run's lists do not wait for it)
@@ -480,7 +482,8 @@ Job set_job(const void* points, const float* ys, int64_t n, int dtype, int32_t* 
 }
 
 int run_set(const Job& j, cudaStream_t stream) {
-  g_launches += (uint64_t)launch_set(j, set_class(j.N), nullptr, 1, false, stream);
+  const int cls = set_class(j.N);
+  g_launches += (uint64_t)launch_set(j, cls, nullptr, 1, cls > 0, false, stream);
   return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
 }
 

@@ -169,8 +169,9 @@ struct SetDesc {
 // there up to kSetOne points.  One CTA per set fills the chip when there are
 // many (600 sets of 16000 points: 0.20 / 0.21 / 0.81 ms on squares, disks and
 // circles, 0.57 / 0.73 / 1.76 in the pipeline); alone it is one SM against all
-// of them: 8000 points take 40 / 50 / 120 us there and 61 / 84 / 216 in the
-// pipeline, 16000 points 63 / 65 / 242 against 63 / 103 / 155.
+// of them: 16000 points take 63 / 65 / 242 us there and 63 / 103 / 155 in the
+// pipeline, so a single set above 1023 points, and those of a batch of few, are
+// split over four CTAs (k_set.cu).
 constexpr int kSetMax = 16383;
 constexpr int kSetOne = 12287;
 constexpr int kSetClasses = 4;
@@ -1152,8 +1153,8 @@ struct Launch {
 
 // Each returns the number of kernels it launched.
 int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
-int launch_set(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st);   // items null: the one set
-int launch_set_list(const Job& j, const Ws& w, cudaStream_t st);   // the sieve's listed points
+int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st);   // items null: the one set
+int launch_set_list(const Job& j, const Ws& w, int sms, cudaStream_t st);   // the sieve's listed points
 SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);
 SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0);
 int launch_table(const Job& j, const Ws& w, cudaStream_t st);

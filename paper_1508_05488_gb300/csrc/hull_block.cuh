@@ -33,9 +33,8 @@ struct BlkSet {
   double ex[4], ey[4];       // the same, as the exact region tests take them
   uint32_t eidx[4];          // candidate numbers of E1..E4
   uint64_t v0[4];            // SPA value of E_r
-  uint64_t klo[4];           // bucket map of region r: by FP32 view (lo, sc), or
-  float lo[4], sc[4];        //   by the sort key's bits (klo, shift)
-  int shift[4];
+  float lo[4], sc[4];        // bucket map of region r
+  uint32_t down;             // exponent that blk_view takes off (word's bits)
   float fA[4], fB[4], fC[4], fE[4];   // FP32 filter of edge r (round1.cuh)
   uint32_t flags;
   int status;
@@ -89,34 +88,37 @@ __device__ __forceinline__ uint32_t blk_word(uint64_t v) {
   return DT == DT_F64 ? (uint32_t)(v >> 32) : (uint32_t)v;
 }
 
+// FP32 view of a sort coordinate for the bucket map.  float64 coordinates of a
+// set beyond 2^60 get 2^-down first, which brings the largest to [1, 2) and
+// what would leave the normal range to 0; non-decreasing in the coordinate.
+template <int DT>
+__device__ __forceinline__ float blk_view(const BlkSet<DT>& s, const typename PT<DT>::T& p, int r) {
+  if constexpr (DT == DT_F64) {
+    uint64_t b = (uint64_t)__double_as_longlong((r & 1) ? p.y : p.x);
+    if (!(s.flags & SF_SMALL)) {
+      const uint32_t h = (uint32_t)(b >> 32);
+      b = (h & 0x7FF00000u) > s.down ? b - ((uint64_t)s.down << 32) : b & 0x8000000000000000ull;
+    }
+    return f64_trunc_f32(b);
+  } else {
+    return __int2float_rn((r & 1) ? p.y : p.x);
+  }
+}
+
 // Bucket of a region-r point, non-decreasing in its sort key.
 template <int DT, int NB>
 __device__ __forceinline__ int blk_bucket(const BlkSet<DT>& s, const typename PT<DT>::T& p, int r) {
-  if (DT == DT_I32 || (s.flags & SF_SMALL)) {
-    float u;
-    if constexpr (DT == DT_F64) u = f64_trunc_f32((uint64_t)__double_as_longlong((r & 1) ? p.y : p.x));
-    else u = __int2float_rn((r & 1) ? p.y : p.x);
-    const float t = __fmul_rn(__fsub_rn(r >= 2 ? -u : u, s.lo[r]), s.sc[r]);
-    return min(max(__float2int_rd(t), 0), NB - 1);
-  }
-  const uint64_t k = blk_key<DT>(p, r);
-  const uint64_t d = k > s.klo[r] ? (k - s.klo[r]) >> s.shift[r] : 0ull;
-  return (int)min(d, (uint64_t)(NB - 1));
+  const float u = blk_view<DT>(s, p, r);
+  const float t = __fmul_rn(__fsub_rn(r >= 2 ? -u : u, s.lo[r]), s.sc[r]);
+  return min(max(__float2int_rd(t), 0), NB - 1);
 }
 
-// Bucket map and SPA seed of region r (e and flags are set).
+// Bucket map and SPA seed of region r (e, flags and down are set).
 template <int DT, int NB>
 __device__ __forceinline__ void blk_map(BlkSet<DT>& s, int r) {
   const typename PT<DT>::T p = s.e[r], q = s.e[(r + 1) & 3];
   s.v0[r] = blk_spa<DT>(p, r);
-  const uint64_t ka = blk_key<DT>(p, r), kb = blk_key<DT>(q, r);
-  const uint64_t span = kb > ka ? kb - ka : 0;
-  s.klo[r] = ka;
-  s.shift[r] = span == 0 ? 0 : max(0, 64 - __clzll((long long)span) - (31 - __clz(NB)));
-  float X, Y, Xn, Yn;
-  f32_view<DT>(p, X, Y);
-  f32_view<DT>(q, Xn, Yn);
-  const float lo = sort_u(X, Y, r), d = __fsub_rn(sort_u(Xn, Yn, r), lo);
+  const float sg = r >= 2 ? -1.f : 1.f, lo = sg * blk_view<DT>(s, p, r), d = __fsub_rn(sg * blk_view<DT>(s, q, r), lo);
   const float sc = d > 0.f ? __fdiv_rn((float)NB, d) : 0.f;
   s.lo[r] = lo;
   s.sc[r] = sc <= 1.0e38f ? sc : 1.0e38f;

@@ -5,9 +5,10 @@
 // the streaming pipeline (nine launches, 80 us for 1000 points), and in a
 // batch its regions would each hold an SM there.
 //
-// Measured (one GB300, us per call): one float64 set of 1000 / 4000 / 8000
-// disk points 21 / 34 / 50 against 63 / 76 / 84 in the pipeline; 4096 float64
-// sets of 256 to 4096 points 224 against 2964.  The exact tests of undecided
+// Measured (one GB300, us per call): one float64 set of 1000 / 3000 / 12000
+// disk points 21 / 24 / 38 (the last two split over four CTAs; 21 / 30 / 55 in
+// one) against 63 / 73 / 92 in the pipeline; 4096 float64 sets of 256 to 4096
+// points 222 against 3080.  The exact tests of undecided
 // points are the costly part: the extremes, which lie on the edges, are let
 // past them (regions of 1000 points: 16k cycles before, 8k after), and one
 // warp runs the last steps alone when few candidates are left (most sets).
@@ -34,9 +35,9 @@ template <>
 struct SetClass<2> { static constexpr int CAP = 4096, T = 256, NB = 512; };
 template <>
 struct SetClass<3> { static constexpr int CAP = 16384, T = 512, NB = 1280; };
-// The sieve's lists of a single set: one CTA per SM in any case, so more warps
-// cost only their barriers (512 -> 1024 threads, us per call: 2M annulus 147 ->
-// 135, 48,007 degenerate points 143 -> 127, 1M int32 square 56 -> 58).
+// Split sets: there is an SM for every CTA, so more warps cost only their
+// barriers (the sieve's lists, 512 -> 1024 threads, us per call: 2M annulus 147
+// -> 135, 48,007 degenerate points 143 -> 127, 1M int32 square 56 -> 58).
 template <>
 struct SetClass<4> { static constexpr int CAP = 16384, T = 1024, NB = 1280; };
 static_assert(SetClass<kSetClasses - 1>::CAP == kSetMax + 1, "the largest class ends at kSetMax");
@@ -55,6 +56,16 @@ struct SetSrc {
 // Order word of a leading word read as FP32, as a signed integer (-0.0 read as +0.0).
 __device__ __forceinline__ int32_t lead_order(float f) { return (int32_t)(f32_order(__fadd_rn(f, 0.0f)) ^ 0x80000000u); }
 
+// Whether p lies strictly outside edge k, exactly.  Out of line: no other value
+// of the caller lives across the test's registers.
+template <int DT>
+__device__ __noinline__ bool set_outside(const BlkSet<DT>& s, uint32_t k, typename PT<DT>::T p, uint32_t flags) {
+  if (flags & (SF_DEGEN0 << k)) return false;
+  const typename PT<DT>::T a = s.e[k], b = s.e[(k + 1) & 3u];
+  if constexpr (DT == DT_F64) return orient_f64(a.x, a.y, b.x, b.y, p.x, p.y) < 0;
+  else return orient_i32(a.x, a.y, b.x, b.y, p.x, p.y, (flags & SF_WIDE) != 0) < 0;
+}
+
 // What k_set works on: the points of whole sets (items, or the one set); a
 // single set's list from the sieve, w.sv_hdr->n points; or the lists of a
 // batch's larger sets, which each CTA first gathers from its set's units.
@@ -63,15 +74,23 @@ enum : int { SET_WHOLE = 0, SET_LIST = 1, SET_BATCH = 2 };
 // float32 vectors (DT_F64 with j.ys) are widened on load.  `beside`: the kernel
 // before this one works on other sets of the same call, so this one starts
 // beside it, and one of its CTAs waits for its end (all of them waiting would
-// hold the SMs: 4096 small float64 sets 246 us, 220 without the overlap).
-// SET_LIST: the listed points (j.pts) are finished by a cluster of four CTAs:
-// each does steps 1-3 on all points and steps 4-7 on one region, whose chain
-// ends in E1..E4, all of them vertices.  The listed points lie close to the
-// hull, so nearly all of them reach the last steps (2300 points of a 20M disk:
-// 57 us in one CTA, 45 of them from the sort on).
-template <int DT, int C, int MODE>
-__global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* items, Ws w, bool beside) {
+// hold the SMs).
+// SPLIT: a set is finished by a cluster of four CTAs: each does step 1 on all
+// points, finds those of one region and does steps 4-7 on them; a region's
+// chain ends in E1..E4, all of them vertices.  The sieve's lists lie close to
+// the hull, so nearly all of their points reach the last steps (2300 points of a
+// 20M disk: 57 us in one CTA, 45 of them from the sort on), and so do those of
+// a circle.  It takes the SMs that a single set or a few leave idle (12,000
+// points, one CTA / split / the pipeline: circle 170 / 61 / 132, beyond 2^60 1051
+// / 213 / 225).
+//
+// 64 registers: what a thread can have where the shared memory of the smaller
+// classes lets the SM fill up (72 and 80, which the exact tests would take:
+// 4096 small float64 sets 306 us against 223).
+template <int DT, int C, int MODE, bool SPLIT>
+__global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(Job j, const SetItem* items, Ws w, bool beside) {
   constexpr bool LIST = MODE == SET_LIST;
+  static_assert(SPLIT || !LIST, "a single set's list is split");
   if (MODE != SET_WHOLE || !beside) griddep_enter();
   if constexpr (LIST) {
     if (!sieved(w)) return;
@@ -87,13 +106,14 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   __shared__ uint32_t red_amin[NW];
   __shared__ int32_t wext[4][NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t part = LIST ? blockIdx.x : 0u;    // LIST: the CTA's region
-  SetItem it = MODE == SET_WHOLE && items ? items[blockIdx.x] : SetItem{0, LIST ? (int32_t)w.sv_hdr->n : (int32_t)j.N, 0};
+  const uint32_t part = SPLIT ? blockIdx.x & 3u : 0u;     // SPLIT: the CTA's region
+  const uint32_t which = SPLIT ? blockIdx.x >> 2 : blockIdx.x;
+  SetItem it = MODE == SET_WHOLE && items ? items[which] : SetItem{0, LIST ? (int32_t)w.sv_hdr->n : (int32_t)j.N, 0};
   if constexpr (MODE == SET_BATCH) {
-    // gather the set's list; a list of another size class, or too long a one
-    // (the pipeline's), is left
-    const SieveSet sv = j.sv_sets[blockIdx.x];
-    if (w.sv_hdr[blockIdx.x].mode == 0) return;
+    // gather the set's list (SPLIT: every CTA of the cluster, the same words);
+    // a list of another size class, or too long a one (the pipeline's), is left
+    const SieveSet sv = j.sv_sets[which];
+    if (w.sv_hdr[which].mode == 0) return;
     const uint32_t* cnt = w.sv_cnt + (size_t)sv.cta0 * kSvWarps;
     static_assert(kSvBatchUnits <= 4 * NB && kSvBatchUnits % T == 0, "the units' prefix fits the table");
     constexpr int PU = kSvBatchUnits / T;
@@ -101,7 +121,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
 #pragma unroll
     for (int q = 0; q < PU; q++) { const int u = tid * PU + q; c[q] = u < sv.nunit ? cnt[u] : 0u; sum += c[q]; }
     uint32_t pre = blk_excl_sum<T>(sum, m.w32[0], total);
-    if (total > (uint32_t)kSetMax || (total < (uint32_t)SetClass<2>::CAP) != (C == 2)) return;
+    if (total > (uint32_t)kSetMax || (!SPLIT && (total < (uint32_t)SetClass<2>::CAP) != (C == 2))) return;
 #pragma unroll
     for (int q = 0; q < PU; q++) { m.tab[tid * PU + q] = pre; pre += c[q]; }
     __syncthreads();
@@ -118,9 +138,9 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
       w.cidx[sv.off + p] = g;
     }
     __syncthreads();
-    it = SetItem{sv.off, (int32_t)total, j.sets[blockIdx.x].id};
-    if (tid == 0) {
-      w.ctl[blockIdx.x].status = ST_SIEVED;
+    it = SetItem{sv.off, (int32_t)total, j.sets[which].id};
+    if (tid == 0 && part == 0) {
+      w.ctl[which].status = ST_SIEVED;
       if (atomicAdd(w.ctr + CT_SIEVE_SETS, 1u) + 1u == (uint32_t)j.nsets) w.ctr[CT_SIEVED] = 1u;
     }
   }
@@ -292,7 +312,11 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
 #pragma unroll
     for (int k = 0; k < 4; k++)
       if (best[k].idx == best[(k + 1) & 3].idx) flags |= SF_DEGEN0 << k;
-    if (lane == 0) { s.flags = flags; s.status = st; }
+    if (lane == 0) {
+      s.flags = flags;
+      s.status = st;
+      s.down = small ? 0u : ((uint32_t)__double2hiint(fmax(xm, ym)) & 0x7FF00000u) - (1023u << 20);
+    }
     __syncwarp();
     if (lane < 4 && st == 0) {
       edge_filter(s.ex[lane], s.ey[lane], s.ex[k1], s.ey[k1], xm, ym, small, s.fA[lane], s.fB[lane], s.fC[lane],
@@ -308,7 +332,10 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   }
   // ---- steps 2-3: the first edge that has the point strictly outside is its
   // region; the FP32 filter decides where it can (round1.cuh), then the exact
-  // test.  Region points are listed and enter the dominance table.
+  // test.  Region points are listed and enter the dominance table.  SPLIT: only
+  // whether it is the CTA's region matters, which it is not for a point inside
+  // the CTA's edge: none of the four tests for a point on another edge, and the
+  // others only for one outside its own.
   {
     float fA[4], fB[4], fC[4], fE[4];
 #pragma unroll
@@ -332,11 +359,14 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
             float X, Y;
             f32_view<DT>(p[u], X, Y);
             uint32_t r = 0;
+            bool in = false;               // SPLIT: certainly inside the CTA's edge
 #pragma unroll
             for (int k = 3; k >= 0; k--) {
               const float d = __fmaf_rn(fA[k], Y, __fmaf_rn(fB[k], X, fC[k]));
               r = !(d > fE[k]) ? (d < -fE[k] ? k + 1 : 8) : r;
+              in |= SPLIT && (uint32_t)k == part && d > fE[k];
             }
+            if (in) r = 0;
             if (r == 8) und |= 1u << u;
             else rr |= r << (4 * u);
           }
@@ -350,9 +380,12 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
         const uint32_t i = (uint32_t)(i0 + u * T + tid);
         if (i == eidx[0] || i == eidx[1] || i == eidx[2] || i == eidx[3]) continue;
         const P p = src.pt(i);
-        uint32_t r;
-        if constexpr (DT == DT_F64) r = (uint32_t)region_exact_f64(p.x, p.y, s.ex, s.ey, flags);
-        else r = (uint32_t)region_exact_i32(p.x, p.y, s.ex, s.ey, flags);
+        uint32_t r = 0;
+        if (!SPLIT || set_outside<DT>(s, part, p, flags)) {
+          for (uint32_t k = 0; k < (SPLIT ? part : 4u) && r == 0; k++)
+            if (set_outside<DT>(s, k, p, flags)) r = k + 1;
+          if (SPLIT && r == 0) r = part + 1;
+        }
         rr |= r << (4 * u);
       }
       uint32_t e[4], take = 0;
@@ -360,7 +393,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
       for (int u = 0; u < 4; u++) {
         const uint32_t i = (uint32_t)(i0 + u * T + tid), r = (rr >> (4 * u)) & 7u;
         e[u] = ((r - 1u) << 14) | i;
-        if (LIST ? r == part + 1u : r != 0) {
+        if (SPLIT ? r == part + 1u : r != 0) {
           const P p = src.pt(i);
           atomicMin(&m.tab[(r - 1) * NB + blk_bucket<DT, NB>(s, p, (int)r - 1)],
                     blk_word<DT>(blk_spa<DT>(p, (int)r - 1)));
@@ -372,7 +405,7 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   }
   __syncthreads();
   uint32_t at = 0;                             // first output slot of the CTA's vertices
-  if constexpr (LIST) {
+  if constexpr (SPLIT) {
     const uint32_t flags = s.flags, all = SF_DEGEN0 * 15u, mine = SF_DEGEN0 << part;
     __syncthreads();
     if (tid == 0) {
@@ -412,54 +445,61 @@ __global__ void __launch_bounds__(SetClass<C>::T) k_set(Job j, const SetItem* it
   if (MODE == SET_WHOLE && beside && blockIdx.x == 0) griddep_enter();
 }
 
-template <int DT, int C, int MODE>
+template <int DT, int C, int MODE, bool SPLIT>
 static void launch_set_c(const Job& j, const SetItem* items, const Ws& w, int count, bool beside, cudaStream_t st) {
   constexpr size_t sm = sizeof(BlkSmem<DT, SetClass<C>::CAP, SetClass<C>::T, SetClass<C>::NB>);
   static bool once = [] {
-    cudaFuncSetAttribute(k_set<DT, C, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_set<DT, C, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     return true;
   }();
   (void)once;
-  launch_pdl_cluster(k_set<DT, C, MODE>, count, SetClass<C>::T, MODE == SET_LIST ? 4 : 1, sm, st, j, items, w, beside);
+  launch_pdl_cluster(k_set<DT, C, MODE, SPLIT>, SPLIT ? 4 * count : count, SetClass<C>::T, SPLIT ? 4 : 1, sm, st, j, items,
+                     w, beside);
 }
 
 template <int DT>
-static void launch_set_t(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st) {
-  if (cls == 0) launch_set_c<DT, 0, SET_WHOLE>(j, items, Ws{}, count, beside, st);
-  else if (cls == 1) launch_set_c<DT, 1, SET_WHOLE>(j, items, Ws{}, count, beside, st);
-  else if (cls == 2) launch_set_c<DT, 2, SET_WHOLE>(j, items, Ws{}, count, beside, st);
-  else launch_set_c<DT, 3, SET_WHOLE>(j, items, Ws{}, count, beside, st);
+static void launch_set_t(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside,
+                         cudaStream_t st) {
+  if (split) launch_set_c<DT, 4, SET_WHOLE, true>(j, items, Ws{}, count, beside, st);
+  else if (cls == 0) launch_set_c<DT, 0, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
+  else if (cls == 1) launch_set_c<DT, 1, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
+  else if (cls == 2) launch_set_c<DT, 2, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
+  else launch_set_c<DT, 3, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
 }
 
 int set_class(int64_t n) {
   return n < SetClass<0>::CAP ? 0 : n < SetClass<1>::CAP ? 1 : n < SetClass<2>::CAP ? 2 : n <= kSetMax ? 3 : -1;
 }
 
-int launch_set(const Job& j, int cls, const SetItem* items, int count, bool beside, cudaStream_t st) {
+int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st) {
   if (count == 0) return 0;
-  if (j.dtype == DT_I32) launch_set_t<DT_I32>(j, cls, items, count, beside, st);
-  else launch_set_t<DT_F64>(j, cls, items, count, beside, st);
+  if (j.dtype == DT_I32) launch_set_t<DT_I32>(j, cls, items, count, split, beside, st);
+  else launch_set_t<DT_F64>(j, cls, items, count, split, beside, st);
   return 1;
 }
 
 template <int DT>
-static int launch_set_list_t(const Job& l, const Ws& w, cudaStream_t st) {
+static int launch_set_list_t(const Job& l, const Ws& w, int sms, cudaStream_t st) {
   if (!l.sv_sets) {
-    launch_set_c<DT, 4, SET_LIST>(l, nullptr, w, 4, false, st);
+    launch_set_c<DT, 4, SET_LIST, true>(l, nullptr, w, 1, false, st);
     return 1;
   }
-  launch_set_c<DT, 2, SET_BATCH>(l, nullptr, w, l.nsets, false, st);
-  launch_set_c<DT, 3, SET_BATCH>(l, nullptr, w, l.nsets, false, st);
+  if (l.nsets <= sms / 4) {
+    launch_set_c<DT, 4, SET_BATCH, true>(l, nullptr, w, l.nsets, false, st);
+    return 1;
+  }
+  launch_set_c<DT, 2, SET_BATCH, false>(l, nullptr, w, l.nsets, false, st);
+  launch_set_c<DT, 3, SET_BATCH, false>(l, nullptr, w, l.nsets, false, st);
   return 2;
 }
 
-int launch_set_list(const Job& j, const Ws& w, cudaStream_t st) {
+int launch_set_list(const Job& j, const Ws& w, int sms, cudaStream_t st) {
   Job l = j;
   l.pts = w.cpts;          // float32 vectors are listed widened
   l.ys = nullptr;
   Ws v = w;
   v.sv_in = j.pts;
-  return j.dtype == DT_I32 ? launch_set_list_t<DT_I32>(l, v, st) : launch_set_list_t<DT_F64>(l, v, st);
+  return j.dtype == DT_I32 ? launch_set_list_t<DT_I32>(l, v, sms, st) : launch_set_list_t<DT_F64>(l, v, sms, st);
 }
 
 }  // namespace cch
