@@ -288,6 +288,7 @@ int copy_tables(Job& j, const Batch& b, Workspace* ws, cudaStream_t stream, bool
     j.sv_sets = reinterpret_cast<const SieveSet*>(dev + sv_off);
     j.sv_cta = reinterpret_cast<const int32_t*>(dev + cta_off);
     j.sv_nctas = (int32_t)b.cta.size();
+    j.sv_all = b.sets.size() <= (size_t)sm_count();
   }
   j.sets = reinterpret_cast<const SetDesc*>(dev + sets_off);
   return CCH_OK;
@@ -377,7 +378,7 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, Works
         cudaEventRecord(rec.sv[k], stream);
     };
     mark_sv(0);
-    nk += launch_table(j, L.w, stream);
+    nk += launch_table(j, L.w, sm_count(), stream);
     mark_sv(1);
     nk += launch_sieve(j, L.w, stream);
     mark_sv(2);
@@ -534,16 +535,24 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
   if (N > 0x7FFFFFFFll) return CCH_ERR_RANGE;
   if (N > 0 && !points) return CCH_ERR_INVALID;
   if ((uintptr_t)points % (dtype == CCH_F64 ? 16 : 8)) return CCH_ERR_INVALID;
+  if (nsets == 1) return cch_hull(points, N, dtype, out_idx, out_counts, stream);   // one set's kernels, not a batch's
   Batch batch;
   const Tune tune = tune_for(dtype, N, nsets);
   int target = a1_target(dtype);
   int64_t len = std::max<int64_t>(tune.a1_len_min, ((N + target - 1) / std::max(target, 1) + 1023) / 1024 * 1024);
   int64_t nch = 0, nt = 0, n3 = 0, np_ = 0;
   const int ct = cls_tile(dtype);
+  int32_t large = 0, sieved = 0;
   for (int32_t s = 0; s < nsets; s++) {
-    int64_t n = offsets[s + 1] - offsets[s];
+    const int64_t n = offsets[s + 1] - offsets[s];
     if (n < 0) return CCH_ERR_INVALID;
     if (n > kMaxSetPoints) return CCH_ERR_RANGE;
+    large += n > (int64_t)kSvBatchFew * kSvBatchLen;
+    sieved += n > kSetMax && n <= (int64_t)kSvBatchFew * kSvBatchLen;
+  }
+  const int32_t units = large >= sm_count() ? kSvBatchUnits : large == 0 || sieved >= kSvBatchSets ? kSvBatchFew : 0;
+  for (int32_t s = 0; s < nsets; s++) {
+    const int64_t n = offsets[s + 1] - offsets[s];
     const int cls = set_class(n);
     if (cls >= 0) {
       batch.items[cls].push_back(SetItem{offsets[s], (int32_t)n, s});
@@ -555,7 +564,7 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
     int32_t cp = (t + kPlanTiles - 1) / kPlanTiles;
     batch.sets.push_back(
         SetDesc{offsets[s], n, (int32_t)nch, c, (int32_t)nt, t, (int32_t)n3, c3, (int32_t)np_, cp, s});
-    const SieveSet sv = sieve_batch_set(offsets[s], n, (int32_t)batch.cta.size());
+    const SieveSet sv = sieve_batch_set(offsets[s], n, (int32_t)batch.cta.size(), units);
     batch.cta.insert(batch.cta.end(), (size_t)(sv.nunit + kSvWarps - 1) / kSvWarps, (int32_t)batch.sieve.size());
     batch.sieve.push_back(sv);
     nch += c;

@@ -143,6 +143,7 @@ enum : int {
   CT_CHAIN_TOTAL,
   CT_OUT_TOTAL,
   CT_SIEVE_SETS,                       // sets of a batch finished by the sieve path
+  CT_SIEVE_NONE,                       // a set of the batch was refused, and so are the others (Job::sv_all)
   CT_SIEVED,                           // the set was finished by the sieve path: the pipeline's kernels leave
   CT_ERR,                              // first device error (negative status)
   CT_COUNT
@@ -184,7 +185,7 @@ struct SetItem {
 // A set of the sieve (k_sieve.cu): nunit units of len consecutive points.
 struct SieveSet {
   int64_t off, n;
-  int64_t cap;          // most points a sieved set may keep (by the sample's estimate)
+  int64_t cap;          // a set of which the sample says that more points are left is refused
   int64_t len;          // points per unit
   int32_t nunit;
   int32_t pre;          // points at the head of every unit that are prefetched
@@ -193,9 +194,17 @@ struct SieveSet {
 };
 constexpr int kSvMaxUnits = 5120;      // of a single set
 constexpr int kSvWarps = 8;            // warps, hence units, per k_sieve CTA
-// A batch's larger sets: units of kSvBatchLen points, kSvBatchUnits per set at
-// most (larger sets take the pipeline), tables of kSvBatchRows bands.
-constexpr int kSvBatchLen = 2048, kSvBatchUnits = 1024, kSvBatchRows = 256;
+// A batch's larger sets: units of kSvBatchLen points, tables of kSvBatchRows
+// bands.  A set's sample has 4096 points, whatever its size, so above kSvBatchFew
+// units its list is long and one CTA's work on it shows unless the batch has such
+// a set for every SM (us per call, sieved / pipeline: 2 float64 squares of 262,144
+// points 84 / 86, of 500,009 103 / 88, of 1,000,003 123 / 92; 16 squares of
+// 1,000,003 285 / 192; 128 disks of 500,009 837 / 962; 1024 int32 sets of up to
+// 2^20 1190 / 1530).  Up to kSvBatchUnits units they are sieved then, otherwise
+// they take the pipeline, and the rest of the batch with them unless it has
+// kSvBatchSets sets to sieve: the two routes one after the other cost more (16 and
+// 64 float64 sets of up to 2^20: 260 and 349 sieved where possible, 150 and 244).
+constexpr int kSvBatchLen = 2048, kSvBatchUnits = 1024, kSvBatchFew = 128, kSvBatchSets = 128, kSvBatchRows = 256;
 // Bands per axis of a single set's tables: of the sample's polygon, and of
 // k_refine's, which has the listed points' own (512 in both: 20M square / disk
 // 144 / 157 us a call, 5M Gaussian 78; 256 and 512: 141 / 152, 73; 256 and
@@ -239,6 +248,7 @@ struct Job {
   const SieveSet* sv_sets;   // a batch: device array beside `sets`, nullptr: no sieve
   const int32_t* sv_cta;     // a batch: set of every k_sieve CTA
   int32_t sv_nctas;
+  uint32_t sv_all;           // a batch: all of its sets are sieved or none
   int32_t* out_idx;     // device
   int32_t* out_counts;  // device, [nsets]
   int32_t* r1_idx;      // stage hook (set 0, or nullptr): round-1 survivors, region-major
@@ -1156,8 +1166,8 @@ int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipel
 int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st);   // items null: the one set
 int launch_set_list(const Job& j, const Ws& w, int sms, cudaStream_t st);   // the sieve's listed points
 SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);
-SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0);
-int launch_table(const Job& j, const Ws& w, cudaStream_t st);
+SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0, int32_t most);
+int launch_table(const Job& j, const Ws& w, int sms, cudaStream_t st);
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st);
 int launch_refine(const Job& j, const Ws& w, cudaStream_t st);   // a single set's; a batch has none
 int launch_extremes(const Job& j, const Ws& w, const Launch& L);

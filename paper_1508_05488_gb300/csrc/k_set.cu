@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(J
     // gather the set's list (SPLIT: every CTA of the cluster, the same words);
     // a list of another size class, or too long a one (the pipeline's), is left
     const SieveSet sv = j.sv_sets[which];
-    if (w.sv_hdr[which].mode == 0) return;
+    if (w.sv_hdr[which].mode == 0 || w.ctr[CT_SIEVE_NONE] != 0) return;
     const uint32_t* cnt = w.sv_cnt + (size_t)sv.cta0 * kSvWarps;
     static_assert(kSvBatchUnits <= 4 * NB && kSvBatchUnits % T == 0, "the units' prefix fits the table");
     constexpr int PU = kSvBatchUnits / T;

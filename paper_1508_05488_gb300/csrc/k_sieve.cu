@@ -55,11 +55,14 @@ namespace {
 
 constexpr int kTabThreads = 1024;                   // of k_refine, and of k_table on a single set
 constexpr int kTabBatchThreads = 256;               // of k_table on a batch's sets: 4096 sample points each, four
-                                                    // sets per SM (512 threads, two: 37 us for 409 sets, 30 so)
+                                                    // sets per SM (512 threads, two: 37 us for 409 sets, 30
+                                                    // so; 1024 where every set has an SM to itself: 5 to 8
+                                                    // us less a call)
 constexpr int kTabItems = 8, kTabBatchItems = 16;   // points per thread at most
 constexpr int kPeel = 40;                           // peeling rounds at most
-constexpr int64_t kLeast = 8;                       // a set of which more than this share and more than kSetMax
-                                                    // points are left is refused
+constexpr int64_t kLeast = 8;                       // where more than this share of a set is left, little of it
+                                                    // lies inside even its own polygon (k_refine)
+constexpr int64_t kSvMost = 131072;                 // points that k_refine takes
 constexpr uint32_t kPlain = 2048;                   // lists up to this size go to k_set as they are
 
 template <int DT>
@@ -411,10 +414,13 @@ __device__ __forceinline__ SieveHdr fresh_hdr(const SieveHdr* h) {
 // with 8 points per thread (8 with 16: 46 us); 131,072 points leave 23,600 of a
 // 20M disk and 5,100 of a square; a sixteenth of the set instead of an eighth
 // changed nothing below 2M points.
-// A set of which the check finds too much left is refused: points on a circle,
-// all left, take 114 / 211 / 258 / 308 / 383 us at 13, 20, 32, 48 and 65 thousand
-// (136 / 235 / 281 / 337 / 414 when k_refine found out); a fifth left (the
-// degenerate kind) is listed up to kSetMax points.
+// A set of which the check finds too much left is refused (found out by k_refine
+// instead, a circle took 23 to 31 us more); a fifth left (the degenerate kind) is
+// listed up to kSetMax points, up to half of that in a batch, whose lists are one
+// CTA's work each where it has many (96 degenerate sets of 60,000: 429 us refused,
+// 787 listed).  A batch with a set per SM at most is sieved whole or not at all
+// (Job::sv_all), so that it does not wait for lists and pipeline in turn (8
+// degenerate sets of 38,000, half of them refused: 314 us, 209 so).
 template <int DT, int R, int CL, int T, int NI>
 __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   griddep_enter();
@@ -445,18 +451,22 @@ __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   // the sample is here: k_sieve's CTAs may start and prefetch
   griddep_release();
   const bool ok = build_table<R, CL, T, NI>(m, X, Y, valid, rank, tab, hdr);
-  // what is left of the first item of every thread tells whether the sieve pays
+  // what is left of the sample (of 16384 points of it, 1024 of a batch's set)
+  // tells whether the sieve pays
+  constexpr int NC = CL > 1 ? 1 : kTabThreads / T;
   uint32_t outn = 0;
   if (ok) {
     const SieveHdr h = fresh_hdr(hdr);
-    outn = (valid & 1u) && !sieve_inside<R, true>(tab, h, X[0], Y[0]);
+#pragma unroll
+    for (int k = 0; k < NC; k++) outn += ((valid >> k) & 1u) && !sieve_inside<R, true>(tab, h, X[k], Y[k]);
     outn = __reduce_add_sync(0xFFFFFFFFu, outn);
     if (lane == 0 && outn) atomicAdd(cl_map<CL>(&m.cnt, 0), outn);
     cl_sync<CL>();
   }
   if (rank == 0 && tid == 0) {
-    const int64_t left = ok ? (int64_t)m.cnt * sd.n / (min(groups, (int64_t)CL * W) * 32) : sd.n;
-    hdr->mode = ok && left <= min(sd.cap, max(sd.n / kLeast, (int64_t)kSetMax)) ? 1u : 0u;
+    const int64_t left = ok ? (int64_t)m.cnt * sd.n / (min(groups, (int64_t)CL * W * NC) * 32) : sd.n;
+    hdr->mode = ok && left <= sd.cap ? 1u : 0u;
+    if (hdr->mode == 0 && j.sv_all) w.ctr[CT_SIEVE_NONE] = 1u;
   }
 }
 
@@ -494,7 +504,7 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
   }
   griddep_enter();
   const SieveHdr hdr = w.sv_hdr[set];
-  if (hdr.mode == 0) return;
+  if (hdr.mode == 0 || w.ctr[CT_SIEVE_NONE] != 0) return;
   for (int i = tid; i < 2 * (R + 2); i += kSvThreads) tab[i] = w.sv_tab[(size_t)set * 2 * (R + 2) + i];
   __syncthreads();
   if (a0 >= sd.n) return;
@@ -724,16 +734,18 @@ bool sieve_fits() {
 }
 
 template <int DT>
-int launch_table_t(const Job& j, const Ws& w, cudaStream_t st) {
+int launch_table_t(const Job& j, const Ws& w, int sms, cudaStream_t st) {
   constexpr int T = kTabThreads, TB = kTabBatchThreads, CL = kSvCluster, R = kSvRows, RB = kSvBatchRows;
-  constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>);
+  constexpr size_t sm = sizeof(TabSmem<R, T>), smb = sizeof(TabSmem<RB, TB>), smf = sizeof(TabSmem<RB, T>);
   if (j.sv_sets) {
     static bool once = [] {
       cudaFuncSetAttribute(k_table<DT, RB, 1, TB, kTabBatchItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb);
+      cudaFuncSetAttribute(k_table<DT, RB, 1, T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smf);
       return true;
     }();
     (void)once;
-    launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
+    if (j.nsets <= sms / 2) launch_pdl(k_table<DT, RB, 1, T, 4>, j.nsets, T, smf, st, j, w);
+    else launch_pdl(k_table<DT, RB, 1, TB, kTabBatchItems>, j.nsets, TB, smb, st, j, w);
     return 1;
   }
   launch_pdl_cluster(k_table<DT, R, CL, T, kTabItems>, CL, T, CL, sm, st, j, w);
@@ -768,25 +780,26 @@ SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms) {
   s.len = ((n + most - 1) / most + step - 1) / step * step;
   s.nunit = (int32_t)((n + s.len - 1) / s.len);
   s.pre = (int32_t)std::min<int64_t>(s.len, kSvPrefetch / ((dtype == DT_F64 ? 16 : 8) * (int64_t)s.nunit));
-  s.cap = kSvCluster * kTabThreads * kTabItems;
+  static_assert(kSvCluster * kTabThreads * kTabItems == kSvMost, "a thread holds kTabItems listed points");
+  s.cap = std::min(kSvMost, std::max<int64_t>(n / kLeast, kSetMax));
   return s;
 }
 
-SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0) {
+SieveSet sieve_batch_set(int64_t off, int64_t n, int32_t cta0, int32_t most) {
   SieveSet s{};
   s.off = off;
   s.n = n;
   s.len = kSvBatchLen;
   const int64_t units = (n + kSvBatchLen - 1) / kSvBatchLen;
-  s.nunit = units <= kSvBatchUnits ? (int32_t)units : 0;
-  s.cap = kSetMax / 4 * 3;
+  s.nunit = units <= most ? (int32_t)units : 0;
+  s.cap = std::min<int64_t>(kSetMax / 4 * 3, std::max<int64_t>(n / kLeast, kSetMax / 2));
   s.cta0 = cta0;
   return s;
 }
 
-int launch_table(const Job& j, const Ws& w, cudaStream_t st) {
-  return j.dtype == DT_F64 ? launch_table_t<DT_F64>(j, w, st)
-         : j.dtype == DT_F32 ? launch_table_t<DT_F32>(j, w, st) : launch_table_t<DT_I32>(j, w, st);
+int launch_table(const Job& j, const Ws& w, int sms, cudaStream_t st) {
+  return j.dtype == DT_F64 ? launch_table_t<DT_F64>(j, w, sms, st)
+         : j.dtype == DT_F32 ? launch_table_t<DT_F32>(j, w, sms, st) : launch_table_t<DT_I32>(j, w, sms, st);
 }
 
 int launch_sieve(const Job& j, const Ws& w, cudaStream_t st) {
