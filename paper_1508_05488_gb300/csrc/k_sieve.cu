@@ -579,7 +579,10 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
 // the listed points themselves where there are more than kPlain (20M disk:
 // 23,600 to 2,300 in 30 us, the steps of k_table again; k_set on the longer list
 // takes more than it saves -- with kPlain at 6144 the 20M square, 5,100 listed,
-// went from 143 to 179 us).
+// went from 143 to 179 us).  Where the sample's polygon left more than a kLeast-th
+// of the set, the listed points lie on the hull's own edge and their polygon drops
+// few of them (degenerate set of 48,007, 9,600 listed: 124 us a call with the
+// polygon, 104 without).
 template <int DT, int R, int CL>
 __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
   griddep_enter();
@@ -628,7 +631,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_refine(Job j, Ws w) {
     }
     return w.valA[sd.off + (int64_t)l * sd.len + (p - m.upre[l])];
   };
-  if (total <= kPlain) {
+  if (total <= kPlain || (total <= (uint32_t)kSetMax && total > sd.n / kLeast)) {
     for (uint32_t i = rank * kTabThreads + tid; i < total; i += CL * kTabThreads) {
       const uint32_t g = listed(i);
       lp[i] = input_point<P>(j, sd.off + g);
