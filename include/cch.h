@@ -205,6 +205,19 @@ int cch_profile_read(double *stage_ms, int max_stages, int64_t *calls);
 uint64_t cch_launch_count(void);
 
 /*
+ * The way that the last call on `stream` that used its workspace took (calls
+ * of small sets use none), for tests and for explaining a timing; synchronises
+ * the stream.  route: host int32[6]
+ *   [0] 1: the one-pass sieve finished every larger set of the call
+ *   [1] sets of a batch that it finished
+ *   [2] regions sorted in shared memory   [3] tiles of the multi-block sort
+ *   [4] runs of equal quantised keys that the multi-block sort put right
+ *   [5] 1: one was too long, and the full sort ran
+ * CCH_ERR_NOTFOUND: the stream has no workspace.
+ */
+int cch_route(void *stream, int32_t *route);
+
+/*
  * Self-test of the device-side failure path: one kernel waits on a device
  * flag that nothing sets, with the same bounded wait every kernel of the
  * library uses, and must give up and report.  Writes to *status_dev (device

@@ -92,6 +92,8 @@ def _load():
         lib.cch_profile_read.argtypes = [vp, ctypes.c_int, vp]
         lib.cch_launch_count.restype = ctypes.c_uint64
         lib.cch_launch_count.argtypes = []
+        lib.cch_route.restype = ctypes.c_int
+        lib.cch_route.argtypes = [vp, vp]
         lib.cch_selftest_wait.restype = ctypes.c_int
         lib.cch_selftest_wait.argtypes = [vp, vp]
         tp = ctypes.POINTER(TuneParams)
@@ -412,6 +414,16 @@ def autotune_batched(points, offsets, out_idx=None, out_counts=None, reps: int =
 def launch_count() -> int:
     """Kernels launched by the library so far."""
     return int(_load().cch_launch_count())
+
+
+ROUTE_NAMES = ("sieved", "sieved_sets", "small_regions", "sort_tiles", "fast_runs", "fast_fail")
+
+
+def route(stream=None) -> dict:
+    """The way of the last call on the stream that used its workspace (synchronises; see cch_route)."""
+    r = np.zeros(len(ROUTE_NAMES), dtype=np.int32)
+    _check(_load().cch_route(_stream_handle(stream), r.ctypes.data), "cch_route")
+    return dict(zip(ROUTE_NAMES, r.tolist()))
 
 
 def workspace_bytes(n: int, dtype_code: int = CCH_F64) -> int:

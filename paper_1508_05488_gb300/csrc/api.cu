@@ -750,6 +750,25 @@ int cch_profile_read(double* stage_ms, int max_stages, int64_t* calls) {
 
 uint64_t cch_launch_count(void) { return g_launches.load(); }
 
+int cch_route(void* stream, int32_t* route) {
+  if (!route) return CCH_ERR_INVALID;
+  cudaStream_t s = (cudaStream_t)stream;
+  std::unique_lock<std::mutex> lk;
+  const std::shared_ptr<Workspace> ws = lock_workspace(s, lk);
+  if (!ws->dev) return CCH_ERR_NOTFOUND;
+  const uint32_t* src = layout(ws->cap, ws->dev).w.ctr;
+  uint32_t c[CT_COUNT];
+  if (cudaMemcpyAsync(c, src, sizeof c, cudaMemcpyDeviceToHost, s) != cudaSuccess) return CCH_ERR_CUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess) return CCH_ERR_CUDA;
+  route[0] = (int32_t)c[CT_SIEVED];
+  route[1] = (int32_t)c[CT_SIEVE_SETS];
+  route[2] = (int32_t)c[CT_SMALL_TOTAL];
+  route[3] = (int32_t)c[CT_SORT_TOTAL];
+  route[4] = (int32_t)c[CT_FAST_RUNS];
+  route[5] = (c[CT_FAST_FAIL] | c[CT_FAST_FAIL2]) != 0;
+  return CCH_OK;
+}
+
 namespace cch {
 namespace {
 // One thread waits on a flag that nothing sets, with the library's bounded
