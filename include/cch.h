@@ -287,9 +287,11 @@ int cch_tune_save(const char *path);
 int cch_tune_load(const char *path);
 /* Measure the choices on this batch (same arguments as cch_hull_batched;
  * device buffers, synchronises the stream): coordinate descent over
- * candidate values of each choice, `reps` timed calls per candidate; the
- * fastest goes into the table under this batch's key and into *best (if not
- * NULL).  The outputs hold the batch's hulls afterwards. */
+ * candidate values of each choice, twice `reps` timed calls per candidate; the
+ * fastest, where it is faster by more than such measurements differ, goes into
+ * the table under this batch's key and into *best (if not NULL).  Where no set
+ * of the batch reaches the pipeline, nothing is searched and the choices stay
+ * as they are.  The outputs hold the batch's hulls afterwards. */
 int cch_autotune_batched(const void *points, const int64_t *offsets, int32_t nsets, int32_t dtype,
                          int32_t *out_idx, int32_t *out_counts, void *stream, int32_t reps,
                          cch_tune_params *best);

@@ -281,8 +281,10 @@ int cch_tune_load(const char* path) {
 
 // Coordinate descent over the candidate values of each choice, timed on the
 // caller's own batch (CUDA events on its stream, one untimed call per
-// candidate first); the fastest choice of every knob is kept in turn.  The
-// result is stored in the table under this call's key and returned.
+// candidate first); a value that is faster by more than two measurements of one
+// value differ is kept, knob by knob.  The result is stored in the table under
+// this call's key and returned.  A batch of which no set reaches the pipeline
+// has nothing to choose from and keeps what it has.
 int cch_autotune_batched(const void* points, const int64_t* offsets, int32_t nsets, int32_t dtype,
                          int32_t* out_idx, int32_t* out_counts, void* stream, int32_t reps,
                          cch_tune_params* best) {
@@ -294,20 +296,40 @@ int cch_autotune_batched(const void* points, const int64_t* offsets, int32_t nse
   cch_tune_params cur;
   int rc = cch_tune_get(nullptr, 0, dtype, batched, bucket, &cur);
   if (rc != CCH_OK && rc != CCH_ERR_NOTFOUND) return rc;
+  bool pipeline = false;
+  for (int32_t s = 0; s < nsets; s++) pipeline |= offsets[s + 1] - offsets[s] > (nsets == 1 ? kSetOne : kSetMax);
+  rc = cch_hull_batched(points, offsets, nsets, dtype, out_idx, out_counts, stream);
+  if (rc != CCH_OK) return rc;
+  if (pipeline) {
+    int32_t route[6];
+    rc = cch_route(stream, route);
+    if (rc != CCH_OK) return rc;
+    pipeline = route[0] == 0;
+  }
+  if (!pipeline) {
+    if (cudaStreamSynchronize(st) != cudaSuccess) return CCH_ERR_CUDA;
+    if (best) *best = cur;
+    return cch_tune_set(nullptr, 0, dtype, batched, bucket, &cur);
+  }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return CCH_ERR_CUDA;
-  auto measure = [&](const cch_tune_params& p, float& ms) -> int {
+  auto measure = [&](const cch_tune_params& p, float& ms, float& spread) -> int {
     int r = cch_tune_set(nullptr, 0, dtype, batched, bucket, &p);
     if (r != CCH_OK) return r;
     r = cch_hull_batched(points, offsets, nsets, dtype, out_idx, out_counts, stream);
     if (r != CCH_OK) return r;
-    cudaEventRecord(e0, st);
-    for (int k = 0; k < reps && r == CCH_OK; k++)
-      r = cch_hull_batched(points, offsets, nsets, dtype, out_idx, out_counts, stream);
-    cudaEventRecord(e1, st);
-    if (r != CCH_OK) return r;
-    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
-      return CCH_ERR_CUDA;
+    float t[2] = {0.f, 0.f};
+    for (float& v : t) {
+      cudaEventRecord(e0, st);
+      for (int k = 0; k < reps && r == CCH_OK; k++)
+        r = cch_hull_batched(points, offsets, nsets, dtype, out_idx, out_counts, stream);
+      cudaEventRecord(e1, st);
+      if (r != CCH_OK) return r;
+      if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&v, e0, e1) != cudaSuccess)
+        return CCH_ERR_CUDA;
+    }
+    ms = std::min(t[0], t[1]);
+    spread = std::max(t[0], t[1]) - ms;
     return CCH_OK;
   };
   const std::vector<int32_t> small_max = {16384, 8192, 4096};
@@ -315,8 +337,8 @@ int cch_autotune_batched(const void* points, const int64_t* offsets, int32_t nse
       {16, 8192, 1 << 20}, {32, 4096, 1 << 19}, {8, 16384, 1 << 21}, {64, 2048, 1 << 18}};
   const std::vector<int32_t> a1_len = {16384, 65536, 262144, 4096};
   const std::vector<int32_t> cls = {2, 1};
-  float best_ms = 0.f;
-  rc = measure(cur, best_ms);
+  float best_ms = 0.f, best_spread = 0.f;
+  rc = measure(cur, best_ms, best_spread);
   for (int knob = 0; knob < 4 && rc == CCH_OK; knob++) {
     const size_t nv = knob == 0 ? small_max.size() : knob == 1 ? stairs.size() : knob == 2 ? a1_len.size()
                                                                                             : cls.size();
@@ -327,9 +349,9 @@ int cch_autotune_batched(const void* points, const int64_t* offsets, int32_t nse
       else if (knob == 2) c.a1_len_min = a1_len[v];
       else c.cls_per_sm = cls[v];
       if (memcmp(&c, &cur, sizeof c) == 0) continue;
-      float ms = 0.f;
-      rc = measure(c, ms);
-      if (rc == CCH_OK && ms < best_ms) { best_ms = ms; cur = c; }
+      float ms = 0.f, spread = 0.f;
+      rc = measure(c, ms, spread);
+      if (rc == CCH_OK && ms + std::max(spread, best_spread) < best_ms) { best_ms = ms; best_spread = spread; cur = c; }
     }
   }
   cudaEventDestroy(e0);
