@@ -393,11 +393,14 @@ EXTRA_CONFIGS = (
 
 def extra_configs_bench(cch, torch, dev, reps, hbm):
     """Mpoints/s, stage times and survivor counts of the degenerate, all-extreme
-    and int32 configurations; for the multi-block sort (k_big) a roofline over
-    the record bytes it moves: one read of the records for the histograms, one
-    read and one write per radix pass actually run (passes whose digit is the
-    same for every record are skipped), the SPA phase's read of every record's
-    index and point and write of the survivors' chain slots."""
+    and int32 configurations, by the route that the timed call took (cch_route);
+    for the multi-block sort (k_big) a roofline over the record bytes it moves.
+    By quantised keys (float64 without a run too long): one read of the 12-byte
+    records, one write of 8-byte ones, a read and a write of those in each of
+    four passes, the check's read.  Full sort: one read of the records for the
+    histograms, one read and one write per radix pass actually run (passes whose
+    digit is the same for every record are skipped).  Then the SPA phase's read
+    of every record's index and point and write of the survivors' chain slots."""
     from paper_1508_05488_gb300 import inputs
     out = {}
     for name, gen, n, dt, desc in EXTRA_CONFIGS:
@@ -417,6 +420,7 @@ def extra_configs_bench(cch, torch, dev, reps, hbm):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / reps
         h = int(cnt.item())
+        route = cch.route()
         cch.profile(True)
         cch.profile_read()
         for _ in range(3):
@@ -428,10 +432,13 @@ def extra_configs_bench(cch, torch, dev, reps, hbm):
         paper = cch.stages(pts, prefilter=False)
         s1 = int(ours["counts"][0])
         s2 = int(ours["counts"][5:9].sum())
-        passes = ours["passes"]
         S = 16 if dt == "f64" else 8
+        big = route["sort_tiles"] > 0
+        fast = big and dt == "f64" and not route["fast_fail"]
+        passes = 4 if fast else ours["passes"] if big else 0
         rec = 12                     # record: 8-byte sort key + 4-byte value
-        big_bytes = rec * s1 + passes * 2 * rec * s1 + (4 + S) * s1 + (S + 4) * s2 if passes else 0
+        sort_bytes = (rec + 8 + passes * 2 * 8 + 8) * s1 if fast else (rec + passes * 2 * rec) * s1
+        big_bytes = sort_bytes + ((8 if fast else 4) + S) * s1 + (S + 4) * s2 if big else 0
         big_ms = st_ms.get("big", 0.0)
         b_alg = hull_alg_bytes(S, n, s1, s2, h)
         entry = {"config": desc, "n": n, "dtype": dt, "ms_per_hull": ms, "mpoints_s": n / ms / 1e3,
@@ -440,9 +447,10 @@ def extra_configs_bench(cch, torch, dev, reps, hbm):
                  "round1_paper": int(paper["counts"][0]), "round1": s1, "spa": s2,
                  "identical_spa_both_modes": all(bool((a == b).all()) and len(a) == len(b)
                                                  for a, b in zip(ours["spa"], paper["spa"])),
-                 "sort_path": "multi-block" if passes else "shared-memory",
+                 "sort_path": "sieve" if route["sieved"] else "multi-block, quantised keys" if fast else
+                              "multi-block" if big else "shared-memory",
                  "radix_passes": passes}
-        if passes and big_ms > 0:
+        if big and big_ms > 0:
             ach = big_bytes / (big_ms * 1e-3) / 1e9
             entry["k_big_roofline"] = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s",
                                        "frac": ach / hbm, "algorithmic_bytes": big_bytes,
@@ -793,7 +801,9 @@ def main():
                 "stage_note": "stage times come from events recorded between the launches, which keep a "
                               "kernel from overlapping the one before (k_sieve prefetches while k_table runs) "
                               "and the pipeline's idle launches from running beside k_set; a hull without "
-                              "events (per_set.*.hull.ms) takes less than the sum of its stages"}
+                              "events (per_set.*.hull.ms) takes less than the sum of its stages.  The "
+                              "k_classify stage holds k_sieve and the pipeline's idle k_classify launch "
+                              "(about 2 us), which kernel_ms_per_launch and frac include"}
     # the whole step against its floor: one read of every input point
     step_bytes = 16.0 * args.n * len(kinds)
     # per set, from the profiled pass (events around every stage): the

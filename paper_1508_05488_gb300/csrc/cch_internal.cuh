@@ -3,7 +3,7 @@
 //
 // Pipeline (Sec. 2.1, steps 1-7), every stage a kernel, every set of points a
 // "set" (a single hull is a batch of one).  Small sets are computed whole by
-// one CTA each (k_set.cu, hull_block.cuh); larger ones go through one pass that
+// one CTA or a cluster of four each (k_set.cu, hull_block.cuh); larger ones go through one pass that
 // drops what a sample's polygon covers (k_sieve.cu); what that refuses, and the
 // stage extraction, takes the pipeline:
 //   a1  k_extremes      four lexicographic extremes + edge set-up (step 1)
@@ -50,7 +50,7 @@ enum : int {
 enum : int { DT_I32 = 1, DT_F64 = 2, DT_F32 = 3 };
 
 // ------------------------------------------------------------------ sizes
-constexpr int kThreads = 256;          // every kernel runs 256-thread CTAs
+constexpr int kThreads = 256;          // CTA size of most pipeline kernels
 constexpr int kWarps = kThreads / 32;
 // a2 tiles (points; a multiple of 32 x kClsConsumers): one TMA stage each
 constexpr int kClsTileF64 = 2048;      // 32 KB
@@ -72,8 +72,7 @@ constexpr int64_t kStairMin = 8192;    // smallest sample of a set
 constexpr int kPlanTiles = 64;         // a2 tiles per survivor-count chunk
 // Gather CTAs per chunk (all of them move a dense chunk): a warp moves its
 // sub-slots one after the other, so few chunks are split finely (circle of 2M
-// points, 16 chunks: 72 us at 8); a batch, with a chunk per small set at least,
-// takes 8.
+// points, 16 chunks: 72 us at 8); with 128 chunks or more, 8.
 constexpr int kGatherSplit = 8, kGatherSplitMax = 64;
 constexpr int kGatherDense = 8192;     // survivors from which a chunk counts as dense
 // a1 reads the last kL2KeepBytes of every set without the evict-first hint,

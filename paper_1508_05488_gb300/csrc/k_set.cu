@@ -1,5 +1,5 @@
 // k_set.cu -- the whole method (Sec. 2.1, steps 1-7) for a small set in one
-// CTA: the four extremes, the region test, and from the region points' list
+// CTA, or in a cluster of four: the four extremes, the region test, and from the region points' list
 // on the block steps of hull_block.cuh.  One launch, no workspace and no
 // dependent kernels: a set of a few thousand points is nothing but latency in
 // the streaming pipeline (nine launches, 80 us for 1000 points), and in a
