@@ -563,10 +563,9 @@ __device__ __forceinline__ bool diff_as_u128(double a, double b, unsigned __int1
 }
 
 // 256-bit product of two magnitudes below 2^118, as four words from the lowest.
-__device__ __forceinline__ void mul_u128(unsigned __int128 a, unsigned __int128 b, uint64_t (&r)[4]) {
-  const uint64_t a0 = (uint64_t)a, a1 = (uint64_t)(a >> 64), b0 = (uint64_t)b, b1 = (uint64_t)(b >> 64);
-  const unsigned __int128 p00 = (unsigned __int128)a0 * b0, p01 = (unsigned __int128)a0 * b1;
-  const unsigned __int128 p10 = (unsigned __int128)a1 * b0, p11 = (unsigned __int128)a1 * b1;
+__device__ __forceinline__ void mul_u128(const uint64_t (&a)[2], const uint64_t (&b)[2], uint64_t (&r)[4]) {
+  const unsigned __int128 p00 = (unsigned __int128)a[0] * b[0], p01 = (unsigned __int128)a[0] * b[1];
+  const unsigned __int128 p10 = (unsigned __int128)a[1] * b[0], p11 = (unsigned __int128)a[1] * b[1];
   const unsigned __int128 mid = (p00 >> 64) + (uint64_t)p01 + (uint64_t)p10;     // < 3 * 2^64
   const unsigned __int128 top = p11 + (p01 >> 64) + (p10 >> 64) + (mid >> 64);   // the product is below 2^236
   r[0] = (uint64_t)p00;
@@ -574,62 +573,70 @@ __device__ __forceinline__ void mul_u128(unsigned __int128 a, unsigned __int128 
   r[2] = (uint64_t)top;
   r[3] = (uint64_t)(top >> 64);
 }
-__device__ __forceinline__ int bitlen_u256(const uint64_t (&r)[4]) {
-  for (int k = 3; k >= 0; k--)
-    if (r[k]) return 64 * k + 64 - __clzll((long long)r[k]);
-  return 0;
-}
 
 // Exact orientation with 128-bit differences, for the triples that the 63-bit
 // ones leave open (one coordinate a thousand times the other in magnitude).
 // Integer pipe only: a warp's expansion below takes 60 us at this part's FP64
-// rate.  False when an exponent gap exceeds 63 bits.
+// rate.  False when an exponent gap exceeds 63 bits.  The loops over the products
+// stay loops: unrolled, the registers that this rare step takes cost its callers
+// spills (k_classify on 16 disks of 2.2M points 205 us, 226 unrolled).
 __device__ __forceinline__ bool orient_f64_wide(double ax, double ay, double bx, double by, double cx, double cy,
                                                 int& sign) {
-  unsigned __int128 m1, m2, m3, m4;
-  int e1, e2, e3, e4, s1, s2, s3, s4;
-  if (!diff_as_u128(ax, cx, m1, e1, s1) || !diff_as_u128(by, cy, m4, e4, s4) || !diff_as_u128(ay, cy, m2, e2, s2) ||
-      !diff_as_u128(bx, cx, m3, e3, s3))
-    return false;
-  const int sl = s1 * s4, sr = s2 * s3;
-  if (sl == 0 || sr == 0 || sl != sr) { sign = sl != 0 ? sl : -sr; return true; }
-  uint64_t l[4], r[4];
-  mul_u128(m1, m4, l);
-  mul_u128(m2, m3, r);
-  const int El = e1 + e4, Er = e2 + e3;
-  const int Ll = bitlen_u256(l) + El, Lr = bitlen_u256(r) + Er;
-  int cmp = Ll > Lr ? 1 : Ll < Lr ? -1 : 0;
-  if (cmp == 0) {
-    // equal lengths: both with the leading bit at the top of 256
-    auto norm = [](uint64_t (&v)[4]) {
-      const int up = 256 - bitlen_u256(v), w = up >> 6, b = up & 63;
-      uint64_t o[4];
+  // (ax - cx)(by - cy) against (ay - cy)(bx - cx)
+  const double d[8] = {ax, cx, by, cy, ay, cy, bx, cx};
+  uint64_t m[4][2], r[2][4];
+  int e[2] = {0, 0}, sg[2] = {1, 1}, up[2];
 #pragma unroll
-      for (int k = 3; k >= 0; k--) {
-        uint64_t hi = 0, lo = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          if (q == k - w) hi = v[q];
-          if (q == k - w - 1) lo = v[q];
-        }
-        o[k] = b ? (hi << b) | (lo >> (64 - b)) : hi;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; k++) v[k] = o[k];
-    };
-    norm(l);
-    norm(r);
-#pragma unroll
-    for (int k = 3; k >= 0; k--)
-      if (cmp == 0) cmp = l[k] > r[k] ? 1 : l[k] < r[k] ? -1 : 0;
+  for (int k = 0; k < 4; k++) {
+    unsigned __int128 q;
+    int ek, sk;
+    if (!diff_as_u128(d[2 * k], d[2 * k + 1], q, ek, sk)) return false;
+    m[k][0] = (uint64_t)q;
+    m[k][1] = (uint64_t)(q >> 64);
+    e[k >> 1] += ek;
+    sg[k >> 1] *= sk;
   }
-  sign = sl > 0 ? cmp : -cmp;
+  if (sg[0] == 0 || sg[1] == 0 || sg[0] != sg[1]) { sign = sg[0] != 0 ? sg[0] : -sg[1]; return true; }
+  // same sign: the products' magnitudes by the place of the leading bit, then
+  // by their words with that bit at the top
+#pragma unroll 1
+  for (int p = 0; p < 2; p++) {
+    mul_u128(m[2 * p], m[2 * p + 1], r[p]);
+    int w = 3;
+    while (r[p][w] == 0) w--;
+    up[p] = 64 * (3 - w) + __clzll((long long)r[p][w]);
+    e[p] -= up[p];
+  }
+  int cmp = e[0] > e[1] ? 1 : e[0] < e[1] ? -1 : 0;
+#pragma unroll 1
+  for (int k = 3; k >= 0 && cmp == 0; k--) {
+    uint64_t v[2];
+#pragma unroll 1
+    for (int p = 0; p < 2; p++) {
+      const int w = k - (up[p] >> 6), b = up[p] & 63;
+      v[p] = w < 0 ? 0 : r[p][w] << b;
+      if (b != 0 && w > 0) v[p] |= r[p][w - 1] >> (64 - b);
+    }
+    cmp = v[0] > v[1] ? 1 : v[0] < v[1] ? -1 : 0;
+  }
+  sign = sg[0] > 0 ? cmp : -cmp;
   return true;
 }
 
+// FP64 filter with Shewchuk's bound (3 + 16 eps) eps (|l| + |r|), eps = 2^-53;
+// false where the sign is open.
+__device__ __forceinline__ bool orient_f64_filter(double ax, double ay, double bx, double by, double cx, double cy,
+                                                  int& sign) {
+  const double l = __dmul_rn(__dsub_rn(ax, cx), __dsub_rn(by, cy));
+  const double r = __dmul_rn(__dsub_rn(ay, cy), __dsub_rn(bx, cx));
+  const double d = __dsub_rn(l, r);
+  const double bound = __dmul_rn(3.3306690738754716e-16, __dadd_rn(fabs(l), fabs(r)));
+  sign = d > bound ? 1 : -d > bound ? -1 : 0;
+  return sign != 0 || (l == 0.0 && r == 0.0);
+}
+
 // Exact sign of the 2x2 determinant where the 63-bit integers do not reach: the
-// 128-bit ones, and for exponent gaps beyond those the FP64 filter with
-// Shewchuk's bound (3 + 16 eps) eps (|l| + |r|), eps = 2^-53, then differences
+// 128-bit ones, and for exponent gaps beyond those the FP64 filter, then differences
 // of expansions (Shewchuk 1997, orient2d): det = (ax-cx)(by-cy) - (ay-cy)(bx-cx).
 // Every difference is split exactly into head + tail, the eight partial
 // products exactly into value + error, and the sixteen terms are summed
@@ -637,14 +644,7 @@ __device__ __forceinline__ bool orient_f64_wide(double ax, double ay, double bx,
 static __device__ __noinline__ int orient_f64_tail(double ax, double ay, double bx, double by, double cx,
                                                   double cy) {
   int sgn;
-  if (orient_f64_wide(ax, ay, bx, by, cx, cy, sgn)) return sgn;
-  const double l = __dmul_rn(__dsub_rn(ax, cx), __dsub_rn(by, cy));
-  const double r = __dmul_rn(__dsub_rn(ay, cy), __dsub_rn(bx, cx));
-  const double d = __dsub_rn(l, r);
-  const double bound = __dmul_rn(3.3306690738754716e-16, __dadd_rn(fabs(l), fabs(r)));
-  if (d > bound) return 1;
-  if (-d > bound) return -1;
-  if (l == 0.0 && r == 0.0) return 0;
+  if (orient_f64_wide(ax, ay, bx, by, cx, cy, sgn) || orient_f64_filter(ax, ay, bx, by, cx, cy, sgn)) return sgn;
   double acx, acxt, bcx, bcxt, acy, acyt, bcy, bcyt;
   ef_two_sum(ax, -cx, acx, acxt);
   ef_two_sum(bx, -cx, bcx, bcxt);
@@ -681,14 +681,18 @@ static __device__ __noinline__ int orient_f64_tail(double ax, double ay, double 
 
 // Exact orientation: the 63-bit integer path when the coordinate differences
 // allow it (close points: the usual case for the near-degenerate triples that
-// reach this point), else the tail above.  Valid for coordinates that are 0 or
-// of magnitude in [2^-400, 2^400] (no underflow or overflow anywhere).  500,009
-// collinear points: 4030 us a hull with the filter and the expansion alone, 171
-// with the 128-bit integers before them.
-__device__ __forceinline__ int orient_f64(double ax, double ay, double bx, double by,
-                                          double cx, double cy) {
+// reach this point), else the FP64 filter (`filter`), which decides most triples
+// of one point beside two that are far apart, then the tail above.  Valid for
+// coordinates that are 0 or of magnitude in [2^-400, 2^400] (no underflow or
+// overflow anywhere).  500,009 collinear points: 4030 us a hull with filter and
+// expansion alone, 151 with the 128-bit integers between them.  Without the filter
+// (k_set on a set beyond 2^60, whose every triple comes here): a circle of 12,000
+// points 219 us, 297 with it; but 48 squares of 5000 points 46, 40 with it.
+__device__ __forceinline__ int orient_f64(double ax, double ay, double bx, double by, double cx, double cy,
+                                          bool filter = true) {
   int sgn;
   if (orient_f64_int(ax, ay, bx, by, cx, cy, sgn)) return sgn;
+  if (filter && orient_f64_filter(ax, ay, bx, by, cx, cy, sgn)) return sgn;
   return orient_f64_tail(ax, ay, bx, by, cx, cy);
 }
 

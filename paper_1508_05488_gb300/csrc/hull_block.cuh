@@ -197,7 +197,7 @@ __device__ __forceinline__ int blk_orient(const typename PT<DT>::T& a, const typ
       o = orient_split_filter(f64_split4(a), f64_split4(b), f64_split4(c));
       if (o) return o;
     }
-    return orient_f64(a.x, a.y, b.x, b.y, c.x, c.y);
+    return orient_f64(a.x, a.y, b.x, b.y, c.x, c.y, flag);
   } else {
     return orient_i32(a.x, a.y, b.x, b.y, c.x, c.y, flag);
   }

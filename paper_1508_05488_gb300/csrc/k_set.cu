@@ -62,7 +62,7 @@ template <int DT>
 __device__ __noinline__ bool set_outside(const BlkSet<DT>& s, uint32_t k, typename PT<DT>::T p, uint32_t flags) {
   if (flags & (SF_DEGEN0 << k)) return false;
   const typename PT<DT>::T a = s.e[k], b = s.e[(k + 1) & 3u];
-  if constexpr (DT == DT_F64) return orient_f64(a.x, a.y, b.x, b.y, p.x, p.y) < 0;
+  if constexpr (DT == DT_F64) return orient_f64(a.x, a.y, b.x, b.y, p.x, p.y, (flags & SF_SMALL) != 0) < 0;
   else return orient_i32(a.x, a.y, b.x, b.y, p.x, p.y, (flags & SF_WIDE) != 0) < 0;
 }
 

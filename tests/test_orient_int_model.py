@@ -37,7 +37,7 @@ def lib(tmp_path_factory):
         pytest.skip("needs g++")
     src = open(os.path.join(ROOT, "paper_1508_05488_gb300", "csrc", "cch_internal.cuh")).read()
     a = src.index("// Exact difference of two float64 values")
-    b = src.index("// Exact sign of the 2x2 determinant where the 63-bit")
+    b = src.index("// FP64 filter with Shewchuk")
     d = tmp_path_factory.mktemp("orient")
     (d / "o.cpp").write_text(SHIM + re.sub(r"#pragma unroll.*", "", src[a:b]) + CALLS)
     so = str(d / "o.so")
