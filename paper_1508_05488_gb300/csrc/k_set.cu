@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(J
     // gather the set's list (SPLIT: every CTA of the cluster, the same words);
     // a list of another size class, or too long a one (the pipeline's), is left
     const SieveSet sv = j.sv_sets[which];
-    if (w.sv_hdr[which].mode == 0 || w.ctr[CT_SIEVE_NONE] != 0) return;
+    if (w.sv_hdr[which].mode == 0 || (j.sv_all && w.ctr[CT_SIEVE_NONE] != 0)) return;
     const uint32_t* cnt = w.sv_cnt + (size_t)sv.cta0 * kSvWarps;
     static_assert(kSvBatchUnits <= 4 * NB && kSvBatchUnits % T == 0, "the units' prefix fits the table");
     constexpr int PU = kSvBatchUnits / T;
@@ -333,9 +333,8 @@ __global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(J
   // ---- steps 2-3: the first edge that has the point strictly outside is its
   // region; the FP32 filter decides where it can (round1.cuh), then the exact
   // test.  Region points are listed and enter the dominance table.  SPLIT: only
-  // whether it is the CTA's region matters, which it is not for a point inside
-  // the CTA's edge: none of the four tests for a point on another edge, and the
-  // others only for one outside its own.
+  // whether it is the CTA's region matters: the CTA's own edge first, and the
+  // earlier ones only for a point outside it.
   {
     float fA[4], fB[4], fC[4], fE[4];
 #pragma unroll
@@ -359,14 +358,11 @@ __global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(J
             float X, Y;
             f32_view<DT>(p[u], X, Y);
             uint32_t r = 0;
-            bool in = false;               // SPLIT: certainly inside the CTA's edge
 #pragma unroll
             for (int k = 3; k >= 0; k--) {
               const float d = __fmaf_rn(fA[k], Y, __fmaf_rn(fB[k], X, fC[k]));
               r = !(d > fE[k]) ? (d < -fE[k] ? k + 1 : 8) : r;
-              in |= SPLIT && (uint32_t)k == part && d > fE[k];
             }
-            if (in) r = 0;
             if (r == 8) und |= 1u << u;
             else rr |= r << (4 * u);
           }

@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(kSvThreads, 4) k_sieve(Job j, Ws w) {
   }
   griddep_enter();
   const SieveHdr hdr = w.sv_hdr[set];
-  if (hdr.mode == 0 || w.ctr[CT_SIEVE_NONE] != 0) return;
+  if (hdr.mode == 0 || (j.sv_all && w.ctr[CT_SIEVE_NONE] != 0)) return;
   for (int i = tid; i < 2 * (R + 2); i += kSvThreads) tab[i] = w.sv_tab[(size_t)set * 2 * (R + 2) + i];
   __syncthreads();
   if (a0 >= sd.n) return;
