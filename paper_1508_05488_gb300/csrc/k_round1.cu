@@ -1625,7 +1625,7 @@ int launch_stairs(const Job& j, const Ws& w, const Launch& L) {
 int launch_gather(const Job& j, const Ws& w, const Launch& L) {
   const int chunks = j.nchunkP < 1 ? 1 : j.nchunkP;
   int split = kGatherSplit;
-  while (split < kGatherSplitMax && chunks * split <= 1024) split *= 2;
+  while (split < kGatherSplitMax && chunks * split * 2 <= 1024) split *= 2;
   launch_pdl(k_gather, chunks * split, kThreads, 0, L.stream, j, w);
   return 1;
 }
