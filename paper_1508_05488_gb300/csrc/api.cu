@@ -385,8 +385,8 @@ int run(Job& j, const Batch* batch, cudaStream_t stream, StageOut* stages, std::
     }
     j.epoch = ws->epoch;
   }
-  if (j.sieve.nunit) j.clear16 = (uint32_t)(L.ctl_bytes / 16);
-  else if (cudaMemsetAsync(ws->dev, 0, L.ctl_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
+  // (a sieved single set's: by k_table)
+  if (!j.sieve.nunit && cudaMemsetAsync(ws->dev, 0, L.ctl_bytes, stream) != cudaSuccess) return CCH_ERR_CUDA;
   if (stages) { j.r1_idx = stages->r1_idx; j.r1_region = stages->r1_region; }
   ProfRec rec{};
   cudaEvent_t* ev = prof_begin(rec);

@@ -248,7 +248,6 @@ struct Job {
   const SieveSet* sv_sets;   // a batch: device array beside `sets`, nullptr: no sieve
   const int32_t* sv_cta;     // a batch: set of every k_sieve CTA
   int32_t sv_nctas;
-  uint32_t clear16;          // 16-byte words from Ws::ctl that k_table clears (a single set; else a memset does)
   uint32_t sv_all;           // a batch: all of its sets are sieved or none
   int32_t* out_idx;     // device
   int32_t* out_counts;  // device, [nsets]

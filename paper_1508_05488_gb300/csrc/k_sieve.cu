@@ -432,8 +432,12 @@ __global__ void __launch_bounds__(T, kTabThreads / T) k_table(Job j, Ws w) {
   const int set = blockIdx.x / CL;
   // a single set's control words: nothing of the call has touched them yet (a
   // memset in front of the kernel: 1 to 2 us more a call)
-  if (rank == 0)
-    for (uint32_t i = tid; i < j.clear16; i += T) reinterpret_cast<uint4*>(w.ctl)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (CL > 1 && rank == 0) {
+    constexpr uint32_t NW = sizeof(SetCtl) / 4;
+    static_assert(sizeof(SetCtl) % 4 == 0, "whole words");
+    for (uint32_t i = tid; i < NW + CT_COUNT; i += T) (i < NW ? reinterpret_cast<uint32_t*>(w.ctl) + i : w.ctr + (i - NW))[0] = 0u;
+    for (uint32_t i = tid; i < (uint32_t)j.nchunkP; i += T) w.ptot[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
   const SieveSet sd = j.sv_sets ? j.sv_sets[set] : j.sieve;
   SieveHdr* hdr = w.sv_hdr + set;
   float4* tab = w.sv_tab + (size_t)set * 2 * (R + 2);
