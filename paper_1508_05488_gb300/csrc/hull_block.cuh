@@ -23,6 +23,8 @@ constexpr int kBlkMax = 16384;          // candidate numbers are below it (14 bi
 // their bucket's best one go first, and a bitonic sort of log2(m)^2 / 2 passes
 // takes the rest.
 constexpr uint32_t kBlkPairs = 128;
+constexpr uint32_t kBlkCrowd = 1024;    // so many candidates are sorted without that (3M int32 square points, some
+                                        // hundred in one bucket: 70 us a call, 73 with it)
 constexpr uint16_t kPin = 0x8000u;      // polygon entry that is one of E1..E4
 
 // Set-wide values of a block, in shared memory.
@@ -531,41 +533,43 @@ __device__ void blk_finish(BlkSmem<DT, CAP, T, NB>& m, const Src& src) {
       // larger index.  Then a bitonic sort of what is left by (region, key, c),
       // the pad entries 0xFFFF last.  (2M points on an 801 x 801 grid, 10,000
       // of them listed from its sides: 316 us a call by the sort alone, 155 so.)
-      for (uint32_t t = tid; t < 4 * NB; t += T) m.tab[t] = 0xFFFFFFFFu;
-      __syncthreads();
-      for (uint32_t t = tid; t < m2; t += T) {
-        const uint32_t e = m.b[t];
-        const int r = (int)(e >> 14);
-        const P p = src.pt(e & 0x3FFFu);
-        const uint64_t v = blk_spa<DT>(p, r), k = blk_key<DT>(p, r);
-        uint32_t* best = &m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
-        uint32_t f = *(volatile uint32_t*)best;
-        for (;;) {
-          if (f != 0xFFFFFFFFu) {
-            const P q = src.pt(f & 0x3FFFu);
-            const uint64_t vf = blk_spa<DT>(q, r), kf = blk_key<DT>(q, r);
-            if (vf < v || (vf == v && (kf < k || (kf == k && f < e)))) break;
+      if (CAP > 2 * kBlkCrowd && m2 > kBlkCrowd) {
+        for (uint32_t t = tid; t < 4 * NB; t += T) m.tab[t] = 0xFFFFFFFFu;
+        __syncthreads();
+        for (uint32_t t = tid; t < m2; t += T) {
+          const uint32_t e = m.b[t];
+          const int r = (int)(e >> 14);
+          const P p = src.pt(e & 0x3FFFu);
+          const uint64_t v = blk_spa<DT>(p, r), k = blk_key<DT>(p, r);
+          uint32_t* best = &m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
+          uint32_t f = *(volatile uint32_t*)best;
+          for (;;) {
+            if (f != 0xFFFFFFFFu) {
+              const P q = src.pt(f & 0x3FFFu);
+              const uint64_t vf = blk_spa<DT>(q, r), kf = blk_key<DT>(q, r);
+              if (vf < v || (vf == v && (kf < k || (kf == k && f < e)))) break;
+            }
+            const uint32_t o = atomicCAS(best, f, e);   // fails only where a better one came
+            if (o == f) break;
+            f = o;
           }
-          const uint32_t o = atomicCAS(best, f, e);   // fails only where a better one came
-          if (o == f) break;
-          f = o;
         }
-      }
-      __syncthreads();
-      for (uint32_t t0 = 0; t0 < m2; t0 += T) {
-        uint32_t e[1] = {0u}, keep = 0;
-        if (t0 + tid < m2) {
-          e[0] = m.b[t0 + tid];
-          const int r = (int)(e[0] >> 14);
-          const P p = src.pt(e[0] & 0x3FFFu);
-          const uint32_t f = m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
-          keep = f == e[0] || blk_key<DT>(p, r) < blk_key<DT>(src.pt(f & 0x3FFFu), r);
+        __syncthreads();
+        for (uint32_t t0 = 0; t0 < m2; t0 += T) {
+          uint32_t e[1] = {0u}, keep = 0;
+          if (t0 + tid < m2) {
+            e[0] = m.b[t0 + tid];
+            const int r = (int)(e[0] >> 14);
+            const P p = src.pt(e[0] & 0x3FFFu);
+            const uint32_t f = m.tab[r * NB + blk_bucket<DT, NB>(s, p, r)];
+            keep = f == e[0] || blk_key<DT>(p, r) < blk_key<DT>(src.pt(f & 0x3FFFu), r);
+          }
+          blk_append(m.a, &m.n[3], keep, e);
         }
-        blk_append(m.a, &m.n[3], keep, e);
+        __syncthreads();
+        m2 = m.n[3];
+        for (uint32_t t = tid; t < m2; t += T) m.b[t] = m.a[t];
       }
-      __syncthreads();
-      m2 = m.n[3];
-      for (uint32_t t = tid; t < m2; t += T) m.b[t] = m.a[t];
       uint32_t N2 = 2;
       while (N2 < m2) N2 <<= 1;
       for (uint32_t t = m2 + tid; t < N2; t += T) m.b[t] = 0xFFFFu;
