@@ -338,7 +338,7 @@ int launch_small_sets(const Job& j, const Batch& b, const SetItem* items, cudaSt
   for (int c = kSetClasses - 1; c >= 0; c--) {
     o -= b.items[c].size();
     const size_t count = b.items[c].size();
-    const bool beside = prev != 0 && prev <= 2 * sms, split = c > 0 && 4 * above <= sms;
+    const bool beside = prev != 0 && prev <= 2 * sms, split = set_splits(j, c) && 4 * above <= sms;
     if (count) prev = split ? 4 * count : count;
     nk += launch_set(j, c, items + o, (int)count, split, beside, stream);
   }
@@ -512,7 +512,7 @@ Job set_job(const void* points, const float* ys, int64_t n, int dtype, int32_t* 
 
 int run_set(const Job& j, cudaStream_t stream) {
   const int cls = set_class(j.N);
-  g_launches += (uint64_t)launch_set(j, cls, nullptr, 1, cls > 0, false, stream);
+  g_launches += (uint64_t)launch_set(j, cls, nullptr, 1, set_splits(j, cls), false, stream);
   return cudaGetLastError() == cudaSuccess ? CCH_OK : CCH_ERR_CUDA;
 }
 

@@ -1166,6 +1166,10 @@ struct Launch {
 };
 
 // Each returns the number of kernels it launched.
+// Whether a set of the class is worth four CTAs where there is room: float64 from
+// 1024 points (2047 disk points 29 / 21 us whole / split), int32, whose tests are
+// integer ones, from 4096 (2371 square points 15 / 16, 8000 21 / 18).
+inline bool set_splits(const Job& j, int cls) { return cls > (j.dtype == DT_I32 ? 2 : 0); }
 int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
 int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st);   // items null: the one set
 int launch_set_list(const Job& j, const Ws& w, int sms, cudaStream_t st);   // the sieve's listed points

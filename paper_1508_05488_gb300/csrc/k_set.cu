@@ -56,14 +56,25 @@ struct SetSrc {
 // Order word of a leading word read as FP32, as a signed integer (-0.0 read as +0.0).
 __device__ __forceinline__ int32_t lead_order(float f) { return (int32_t)(f32_order(__fadd_rn(f, 0.0f)) ^ 0x80000000u); }
 
-// Whether p lies strictly outside edge k, exactly.  Out of line: no other value
-// of the caller lives across the test's registers.
+// Whether p lies strictly outside edge k, exactly; and the first edge that has it
+// outside (1..4, 0: none; int32: region_exact_i32).  Out of line: no other value of
+// the caller lives across the tests' registers.
 template <int DT>
-__device__ __noinline__ bool set_outside(const BlkSet<DT>& s, uint32_t k, typename PT<DT>::T p, uint32_t flags) {
+__device__ __forceinline__ bool set_outside_in(const BlkSet<DT>& s, uint32_t k, const typename PT<DT>::T& p, uint32_t flags) {
   if (flags & (SF_DEGEN0 << k)) return false;
   const typename PT<DT>::T a = s.e[k], b = s.e[(k + 1) & 3u];
   if constexpr (DT == DT_F64) return orient_f64(a.x, a.y, b.x, b.y, p.x, p.y, (flags & SF_SMALL) != 0) < 0;
   else return orient_i32(a.x, a.y, b.x, b.y, p.x, p.y, (flags & SF_WIDE) != 0) < 0;
+}
+template <int DT>
+__device__ __noinline__ bool set_outside(const BlkSet<DT>& s, uint32_t k, typename PT<DT>::T p, uint32_t flags) {
+  return set_outside_in<DT>(s, k, p, flags);
+}
+static __device__ __noinline__ uint32_t set_region(const BlkSet<DT_F64>& s, double2 p, uint32_t flags) {
+#pragma unroll 1
+  for (uint32_t k = 0; k < 4u; k++)
+    if (set_outside_in<DT_F64>(s, k, p, flags)) return k + 1;
+  return 0;
 }
 
 // What k_set works on: the points of whole sets (items, or the one set); a
@@ -377,10 +388,13 @@ __global__ void __launch_bounds__(SetClass<C>::T, 1024 / SetClass<C>::T) k_set(J
         if (i == eidx[0] || i == eidx[1] || i == eidx[2] || i == eidx[3]) continue;
         const P p = src.pt(i);
         uint32_t r = 0;
-        if (!SPLIT || set_outside<DT>(s, part, p, flags)) {
-          for (uint32_t k = 0; k < (SPLIT ? part : 4u) && r == 0; k++)
+        if constexpr (!SPLIT) {
+          if constexpr (DT == DT_F64) r = set_region(s, p, flags);
+          else r = (uint32_t)region_exact_i32(p.x, p.y, s.ex, s.ey, flags);
+        } else if (set_outside<DT>(s, part, p, flags)) {
+          for (uint32_t k = 0; k < part && r == 0; k++)
             if (set_outside<DT>(s, k, p, flags)) r = k + 1;
-          if (SPLIT && r == 0) r = part + 1;
+          if (r == 0) r = part + 1;
         }
         rr |= r << (4 * u);
       }

@@ -324,4 +324,16 @@ static __device__ __noinline__ int region_exact_i32_wide(int px, int py, const d
   return 0;
 }
 
+// The same with 64-bit products where the set's spans allow them.
+static __device__ __noinline__ int region_exact_i32(int px, int py, const double* ex, const double* ey,
+                                                    uint32_t flags) {
+  if (flags & SF_WIDE) return region_exact_i32_wide(px, py, ex, ey, flags);
+  for (int k = 0; k < 4; k++) {
+    if (flags & (SF_DEGEN0 << k)) continue;
+    const int k1 = (k + 1) & 3;
+    if (orient_i32((int)ex[k], (int)ey[k], (int)ex[k1], (int)ey[k1], px, py, false) < 0) return k + 1;
+  }
+  return 0;
+}
+
 }  // namespace cch
