@@ -570,15 +570,21 @@ int cch_hull_batched(const void* points, const int64_t* offsets, int32_t nsets, 
   int64_t len = std::max<int64_t>(tune.a1_len_min, ((N + target - 1) / std::max(target, 1) + 1023) / 1024 * 1024);
   int64_t nch = 0, nt = 0, n3 = 0, np_ = 0;
   const int ct = cls_tile(dtype);
-  int32_t large = 0, sieved = 0;
+  int32_t small[kSetClasses] = {}, larger = 0, large = 0;   // k_set's by class, others, those above the sieve of few
   for (int32_t s = 0; s < nsets; s++) {
     const int64_t n = offsets[s + 1] - offsets[s];
     if (n < 0) return CCH_ERR_INVALID;
     if (n > kMaxSetPoints) return CCH_ERR_RANGE;
+    const int cls = set_class(n);
+    if (cls >= 0) small[cls]++;
+    else larger++;
     large += n > (int64_t)kSvBatchFew * kSvBatchLen;
-    sieved += n > kSetMax && n <= (int64_t)kSvBatchFew * kSvBatchLen;
   }
-  const int32_t units = large >= sm_count() ? kSvBatchUnits : large == 0 || sieved >= kSvBatchSets ? kSvBatchFew : 0;
+  for (int c = 0; c < kSetClasses; c++) batch.items[c].reserve(small[c]);
+  batch.sets.reserve(larger);
+  batch.sieve.reserve(larger);
+  const int32_t units =
+      large >= sm_count() ? kSvBatchUnits : large == 0 || larger - large >= kSvBatchSets ? kSvBatchFew : 0;
   for (int32_t s = 0; s < nsets; s++) {
     const int64_t n = offsets[s + 1] - offsets[s];
     const int cls = set_class(n);

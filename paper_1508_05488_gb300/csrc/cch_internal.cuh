@@ -176,6 +176,7 @@ struct SetDesc {
 constexpr int kSetMax = 16383;
 constexpr int kSetOne = 12287;
 constexpr int kSetClasses = 4;
+constexpr int kSetCap[kSetClasses] = {1024, 2048, 4096, kSetMax + 1};   // sets of fewer points, by class
 struct SetItem {
   int64_t off;          // first point, and first output slot
   int32_t n;
@@ -1150,8 +1151,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // words it leaves are not ready to any of them.
 constexpr uint32_t kEpochLast = 0xFFEu, kEpochGraph = 0xFFFu;
 
-// Whether the stream is being captured into a graph.
+// Whether the stream is being captured into a graph (the legacy default stream
+// cannot be).
 inline bool capturing(cudaStream_t st) {
+  if (st == nullptr || st == cudaStreamLegacy) return false;
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { cudaGetLastError(); return false; }
   return s == cudaStreamCaptureStatusActive;
@@ -1170,7 +1173,10 @@ struct Launch {
 // 1024 points (2047 disk points 29 / 21 us whole / split), int32, whose tests are
 // integer ones, from 4096 (2371 square points 15 / 16, 8000 21 / 18).
 inline bool set_splits(const Job& j, int cls) { return cls > (j.dtype == DT_I32 ? 2 : 0); }
-int set_class(int64_t n);   // size class of k_set, or -1 for a set of the pipeline
+// Size class of k_set, or -1 for a set of the pipeline.
+inline int set_class(int64_t n) {
+  return n < kSetCap[0] ? 0 : n < kSetCap[1] ? 1 : n < kSetCap[2] ? 2 : n < kSetCap[3] ? 3 : -1;
+}
 int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st);   // items null: the one set
 int launch_set_list(const Job& j, const Ws& w, int sms, cudaStream_t st);   // the sieve's listed points
 SieveSet sieve_set(int64_t off, int64_t n, int dtype, int sms);

@@ -40,7 +40,8 @@ struct SetClass<3> { static constexpr int CAP = 16384, T = 512, NB = 1280; };
 // -> 135, 48,007 degenerate points 143 -> 127, 1M int32 square 56 -> 58).
 template <>
 struct SetClass<4> { static constexpr int CAP = 16384, T = 1024, NB = 1280; };
-static_assert(SetClass<kSetClasses - 1>::CAP == kSetMax + 1, "the largest class ends at kSetMax");
+static_assert(SetClass<0>::CAP == kSetCap[0] && SetClass<1>::CAP == kSetCap[1] && SetClass<2>::CAP == kSetCap[2] &&
+              SetClass<3>::CAP == kSetCap[3] && SetClass<4>::CAP == kSetCap[3], "the classes of set_class");
 
 // Point c of the set, and the index it is reported as: its own, or that of the
 // sieve's list (`map`).
@@ -475,10 +476,6 @@ static void launch_set_t(const Job& j, int cls, const SetItem* items, int count,
   else if (cls == 1) launch_set_c<DT, 1, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
   else if (cls == 2) launch_set_c<DT, 2, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
   else launch_set_c<DT, 3, SET_WHOLE, false>(j, items, Ws{}, count, beside, st);
-}
-
-int set_class(int64_t n) {
-  return n < SetClass<0>::CAP ? 0 : n < SetClass<1>::CAP ? 1 : n < SetClass<2>::CAP ? 2 : n <= kSetMax ? 3 : -1;
 }
 
 int launch_set(const Job& j, int cls, const SetItem* items, int count, bool split, bool beside, cudaStream_t st) {
