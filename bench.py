@@ -34,7 +34,7 @@ NCU_TRAFFIC = {
     # kernel: (bytes per point, source file, src_sha1 of that file when captured)
     # mean over the three 20M float64 sets (one-pass dram__bytes_read.sum +
     # dram__bytes_write.sum per launch, cold caches)
-    "k_sieve": (16.1899, "paper_1508_05488_gb300/csrc/k_sieve.cu", "650d053710df4c0bb5055fe4f87da968cf8460de"),
+    "k_sieve": (16.1846, "paper_1508_05488_gb300/csrc/k_sieve.cu", "3b4a713b41b894dc8289fc1192f93476a22767ce"),
 }
 
 

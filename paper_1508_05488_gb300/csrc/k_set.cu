@@ -6,9 +6,9 @@
 // batch its regions would each hold an SM there.
 //
 // Measured (one GB300, us per call): one float64 set of 1000 / 3000 / 12000
-// disk points 21 / 24 / 38 (the last two split over four CTAs; 21 / 30 / 55 in
-// one) against 63 / 73 / 92 in the pipeline; 4096 float64 sets of 256 to 4096
-// points 222 against 3080.  The exact tests of undecided
+// disk points 20 / 22 / 36 (the last two split over four CTAs; 29 / 54 in one)
+// against 62 / 72 / 93 in the pipeline; 4096 float64 sets of 256 to 4096
+// points 212 against 3092.  The exact tests of undecided
 // points are the costly part: the extremes, which lie on the edges, are let
 // past them (regions of 1000 points: 16k cycles before, 8k after), and one
 // warp runs the last steps alone when few candidates are left (most sets).
@@ -93,8 +93,8 @@ enum : int { SET_WHOLE = 0, SET_LIST = 1, SET_BATCH = 2 };
 // the hull, so nearly all of their points reach the last steps (2300 points of a
 // 20M disk: 57 us in one CTA, 45 of them from the sort on), and so do those of
 // a circle.  It takes the SMs that a single set or a few leave idle (12,000
-// points, one CTA / split / the pipeline: circle 170 / 61 / 132, beyond 2^60 1051
-// / 213 / 225).
+// points, one CTA / split / the pipeline: circle 166 / 59 / 134, beyond 2^60 1025
+// / 218 / 225).
 //
 // 64 registers: what a thread can have where the shared memory of the smaller
 // classes lets the SM fill up (72 and 80, which the exact tests would take:
